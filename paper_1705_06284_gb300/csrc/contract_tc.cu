@@ -24,10 +24,10 @@
 //   * every 1,024 points the producers read the accumulators back
 //     (tcgen05.ld) into compensated (Kahan) FP32 sums per item in shared
 //     memory, after the next step's operands are handed off.
-// An MMA of M = 128 and K = 16 occupies the issuing thread for about 100
-// cycles whatever N is up to 160 (measured), so the fewer and wider the MMAs
-// the better; the producers run up to three steps ahead of them (operand-B
-// ring of up to 4 stages).  In a single-tile trispectrum pass the inner pair
+// An MMA of M = 128 and K = 16 takes N / 2 cycles of the tensor pipe and, issued
+// under elect.sync, no more of the issuing thread (measured, N = 32..256); the
+// producers run up to three steps ahead of them (operand-B ring of up to 4
+// stages).  In a single-tile trispectrum pass the inner pair
 // rows that are outer rows too are stored into operand B by the operand-A
 // warps that form the same products.
 // Each CTA owns a contiguous range of points; its sums go to its own row of
@@ -163,6 +163,17 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
 // kind::f16 instruction descriptor: BF16 A and B, FP32 D, both K-major.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// One lane of a converged warp (the same lane each time).  Code under
+// elect.sync is known to run on one thread, so the descriptors of its MMAs go
+// to uniform registers once; under an ordinary `lane == 0` branch every
+// tcgen05.mma costs the issuing thread at least 45 cycles, under elect.sync
+// N / 2 (the tensor pipe's own rate at M = 128, K = 16), measured for N = 32..256.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok));
+    return ok != 0;
 }
 
 __device__ __forceinline__ void mma_commit(uint64_t *bar) {
@@ -544,7 +555,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
     if (warp == kLoadWarp) {
         // ================= field loader (one thread) =================
-        if (lane == 0 && c0 < c1) {
+        if (elect_one() && c0 < c1) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&fmap)) : "memory");
             const uint32_t bytes = 2u * KA * (uint32_t)nbins * 128u;
             Ring<NSTG> rs;
@@ -575,7 +586,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
     } else if (warp == kMmaWarp) {
         // ================= MMA issuer (one thread) =================
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = idesc_bf16(128, Npad);
             const uint32_t idesc2 = idesc_bf16(128, 2 * Npad);  // hi and lo rows of B together
             Ring<NST> ra;
@@ -949,7 +960,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
 
     if (warp == kWideProd) {
         // ================= MMA issuer =================
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = idesc_bf16(128, Ng);
             long long g = 0, nfl = 0;
             bool fresh = true;
