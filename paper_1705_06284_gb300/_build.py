@@ -18,7 +18,7 @@ INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(HERE, "libfbs.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
-SOURCES = ["plan.cpp", "pair_cover.cpp", "levels.cpp", "fft.cu", "contract.cu", "contract_tc.cu", "rebin.cu",
+SOURCES = ["plan.cpp", "pair_cover.cpp", "gram_rows.cpp", "levels.cpp", "fft.cu", "contract.cu", "contract_tc.cu", "contract_gram.cu", "rebin.cu",
            "quad_counts.cu", "diagonal.cu", "general.cu",
            "noalloc.cu"]
 

@@ -54,6 +54,7 @@
 
 #include "fbs_internal.h"
 #include "pair_cover.h"
+#include "tc_ptx.cuh"
 
 namespace fbs {
 
@@ -61,7 +62,6 @@ namespace {
 
 constexpr int KC = 64;              // points per chunk (one 128-byte swizzle row of BF16)
 constexpr int kStageLd = KC + 4;    // staged row stride in floats (bank spread)
-constexpr long long kWaitCycles = 2000000000LL;
 
 constexpr int kMaxInner = 256;       // operand-B rows (N of the MMA) at most
 
@@ -109,44 +109,6 @@ struct TcState {
     int *d_err = nullptr;     // the root plan's flags: [0] this evaluation's wait-timeout code, [1] sticky copy
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Wait for the phase of the given parity; false on timeout.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
-    long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity)) {
-        if (clock64() - t0 > kWaitCycles) return false;
-    }
-    return true;
-}
-
-__device__ __forceinline__ void fence_proxy_async_smem() {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-
 // K-major, 128-byte swizzled operand tile: rows of 128 B (64 BF16 along K),
 // 8-row groups 1024 B apart.  Start address must sit in a 1024-B aligned tile
 // (plus the 32-B K-step offset).
@@ -163,23 +125,6 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
 // kind::f16 instruction descriptor: BF16 A and B, FP32 D, both K-major.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-// One lane of a converged warp (the same lane each time).  Code under
-// elect.sync is known to run on one thread, so the descriptors of its MMAs go
-// to uniform registers once; under an ordinary `lane == 0` branch every
-// tcgen05.mma costs the issuing thread at least 45 cycles, under elect.sync
-// N / 2 (the tensor pipe's own rate at M = 128, K = 16), measured for N = 32..256.
-__device__ __forceinline__ bool elect_one() {
-    uint32_t ok;
-    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok));
-    return ok != 0;
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                     smem_u32(bar))
-                 : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float *v) {
@@ -264,45 +209,6 @@ struct TcBars {
     uint64_t full[kMaxAStages], empty[kMaxAStages], bfull[kMaxBStages], bempty[kMaxBStages], accr, accf;
 };
 
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-// 2-D tiled TMA load (x = point, y = bin) into shared memory; completion is
-// counted in bytes on the mbarrier.  Points past the tensor's end read zero.
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y,
-                                            uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-        "[%4];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-        : "memory");
-}
-
-// Bounded wait that gives up at once after any other wait of the CTA timed
-// out (the abort flag is sticky), so no role can strand another.
-// `limit` is the launch's hand-off wait limit in clock cycles (about one
-// second by default; a plan option shortens it to exercise this path).
-__device__ __forceinline__ bool role_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
-                                          int *err, int code, long long limit) {
-    if (mbar_try_wait(bar, parity)) return true;  // ready: no clock read, no flag read
-    long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity)) {
-        if (*abort_flag) return false;
-        if (clock64() - t0 > limit) {
-            *abort_flag = 1;
-            atomicExch(err, code);
-            return false;
-        }
-    }
-    return true;
-}
-
 // Position in a ring of S slots: the slot and the parity of its use count
 // (the phase a consumer waits for; a producer refilling the slot waits for
 // the opposite parity once every slot has been used).
@@ -357,16 +263,6 @@ __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_
             " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
             "r"(a_tmem), "l"(b), "r"(idesc)
             : "memory");
-}
-
-// Compensated (Kahan) FP32 running sum: x = sum, y = compensation; the
-// value is x - y.  Explicit round-to-nearest operations keep the compiler
-// from contracting or reassociating them.
-__device__ __forceinline__ void kahan_add(float2 &a, float v) {
-    const float y = __fsub_rn(v, a.y);
-    const float t = __fadd_rn(a.x, y);
-    a.y = __fsub_rn(__fsub_rn(t, a.x), y);
-    a.x = t;
 }
 
 // A field stage holds 64 KA points of every bin as 2 KA boxes of 32 points,
@@ -1334,6 +1230,12 @@ static void attach_feed(Plan &p, TcJob &job, const std::vector<TcPair> &hp, cons
     FBS_CUDA(cudaStreamSynchronize(p.stream));
 }
 
+// FP64 partial rows of a fused pass (once per level).
+static void fused_partials(Plan &p) {
+    if (p.d_fpart) return;
+    p.d_fpart = (double *)p.dalloc((size_t)p.part_blocks * (p.ttask.nitems + p.qtask.nitems) * sizeof(double));
+}
+
 // The triplets and quadruplets of a trispectrum plan as one contraction over
 // the same shell fields: outer rows are the union of the triplets' pairs
 // (b, c) and the quadruplets' pairs (c, d); inner rows are the triplets'
@@ -1456,8 +1358,7 @@ static void build_fused_job(Plan &p, TcJob &job) {
         hp.push_back(q);
     }
     finish_job(p, job, hp, inner, iout);
-    if (job.usable)
-        p.d_fpart = (double *)p.dalloc((size_t)p.part_blocks * (tt.nitems + qt.nitems) * sizeof(double));
+    if (job.usable) fused_partials(p);
     if (job.usable) attach_feed(p, job, hp, inner, nbuild);
 }
 
@@ -1564,6 +1465,7 @@ static bool launch_wide(Plan &p, const float *islab, long long npts, long long s
 // and of its latest launch the merged flag and points per step / 64.
 void tc_job_info(Plan &p, int which, int32_t *out) {
     for (int i = 0; i < 11; ++i) out[i] = 0;
+    if (which != 1 && p.gram && gram_usable(p, which == 2) && gram_job_info(p, which == 2, out)) return;
     if (!p.tc) return;
     TcState &st = *reinterpret_cast<TcState *>(p.tc);
     const TcJob &j = which == 0 ? st.trip : which == 1 ? st.quad : st.fused;
@@ -1589,43 +1491,6 @@ bool tc_quads_usable(Plan &p) {
     if (st.wquad.usable) return true;
     if (!st.quad.built) build_job(p, p.qtask, true, st.quad);
     return st.quad.usable;
-}
-
-// cuTensorMapEncodeTiled through cudaGetDriverEntryPointByVersion, so the
-// library links only the CUDA runtime (not libcuda directly).
-static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            f = nullptr;
-        return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
-    }();
-    return fn;
-}
-
-// Tensor map of one slab of shell fields: x = point (npts valid, contiguous),
-// y = bin (stride slab_stride floats); boxes of 32 points x all bins in the
-// 128-byte swizzle; points past npts read as zero.
-static CUtensorMap field_tensor_map(const float *islab, long long npts, long long slab_stride, int nbins,
-                                    int rows) {
-    auto enc = tensor_map_encoder();
-    if (!enc) throw Failure{FBS_ERR_CUDA, "cuTensorMapEncodeTiled is not available"};
-    if ((reinterpret_cast<uintptr_t>(islab) & 15) || ((slab_stride * 4) & 15) || nbins < 1 || nbins > 256 ||
-        rows < nbins || npts < 1 || npts >= (1LL << 31))
-        throw Failure{FBS_ERR_ARG, "shell-field slab does not meet the TMA layout rules"};
-    CUtensorMap m;
-    cuuint64_t dims[2] = {(cuuint64_t)npts, (cuuint64_t)rows};  // rows: nbins per field of a batch
-    cuuint64_t strides[1] = {(cuuint64_t)slab_stride * 4};
-    cuuint32_t box[2] = {32u, (cuuint32_t)nbins};
-    cuuint32_t es[2] = {1u, 1u};
-    CUresult r = enc(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(islab), dims, strides, box, es,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) throw Failure{FBS_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")"};
-    return m;
 }
 
 static void launch_job(Plan &p, TcJob &job, const float *islab, long long npts, long long slab_stride,
@@ -1696,7 +1561,7 @@ static void launch_job(Plan &p, TcJob &job, const float *islab, long long npts, 
     if (!pick(want_nsb)) pick(0);
     const size_t sm = tc_smem_bytes(p.nbins, job.Npad, sums, job.maxtiles, nstg, ka, nsb);
     const int flush_every = 16 / ka;  // 1024 points in FP32 per flush
-    const CUtensorMap fmap = field_tensor_map(islab, npts, slab_stride, p.nbins, nf * p.nbins);
+    const CUtensorMap fmap = field_map(islab, npts, slab_stride, p.nbins, nf * p.nbins, 32, true);
     KTimer tm(p, kclass);
     dim3 grid(G, ngrp, nf);
     job.last_merged = stacked ? 2 : merged;
@@ -1742,6 +1607,10 @@ void launch_contract_tc(Plan &p, const float *islab, long long npts, long long s
                         int nf, double *part) {
     const TaskList &t = quads ? p.qtask : p.ttask;
     if (t.nitems == 0) return;
+    if (!quads && gram_usable(p, false)) {
+        launch_gram(p, false, islab, npts, slab_stride, part ? part : p.d_tpart, t.nitems, KC_CONTRACT_TC, nf);
+        return;
+    }
     if (nf == 1 && launch_wide(p, islab, npts, slab_stride, quads)) return;  // batches: narrow only
     TcState &st = tc_state(p);
     TcJob &job = quads ? st.quad : st.trip;
@@ -1755,6 +1624,10 @@ void launch_contract_tc(Plan &p, const float *islab, long long npts, long long s
 
 bool tc_fused_usable(Plan &p) {
     if (p.tc_wide || p.ttask.nitems == 0 || p.qtask.nitems == 0) return false;
+    if (gram_usable(p, true)) {
+        fused_partials(p);
+        return true;
+    }
     TcState &st = tc_state(p);
     if (st.fused.built && st.fused.variant != p.tc_pairs) st.fused = TcJob{};  // option changed: rebuild
     if (!st.fused.built) build_fused_job(p, st.fused);
@@ -1762,6 +1635,10 @@ bool tc_fused_usable(Plan &p) {
 }
 
 void launch_contract_tc_fused(Plan &p, const float *islab, long long npts, long long slab_stride) {
+    if (gram_usable(p, true)) {
+        launch_gram(p, true, islab, npts, slab_stride, p.d_fpart, p.ttask.nitems + p.qtask.nitems, KC_QUAD_TC, 1);
+        return;
+    }
     TcState &st = tc_state(p);
     launch_job(p, st.fused, islab, npts, slab_stride, p.d_fpart, p.ttask.nitems + p.qtask.nitems,
                KC_QUAD_TC, 1);

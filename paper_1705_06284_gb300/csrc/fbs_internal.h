@@ -139,6 +139,14 @@ bool tc_quads_usable(Plan &p);
 // Triplets and quadruplets of a trispectrum plan in one tensor-core pass.
 bool tc_fused_usable(Plan &p);
 void launch_contract_tc_fused(Plan &p, const float *islab, long long npts, long long slab_stride);
+// contract_gram.cu: the shared-operand tensor-core contraction (BF16x3, every
+// tensor-core option at its default), for the triplets of a level or (fused)
+// its triplets and quadruplets together
+bool gram_usable(Plan &p, bool fused);
+void launch_gram(Plan &p, bool fused, const float *islab, long long npts, long long slab_stride, double *part,
+                 int nitems_total, int kclass, int nf);
+bool gram_job_info(Plan &p, bool fused, int32_t *out);
+void free_gram_state(Plan &p);
 void launch_level_reduce(Plan &level, bool quads);
 void launch_level_reduce_batch(Plan &level, bool quads, int nf, const double *tpart, const double *sq,
                                double *tnum, double *sumsq);
@@ -265,6 +273,8 @@ struct Plan {
     long long *d_shell = nullptr;
     // tensor-core path
     void *tc = nullptr;           // opaque state of contract_tc.cu
+    void *gram = nullptr;         // opaque state of contract_gram.cu
+    bool gram_off = false;        // level: this evaluation contracts through tensor memory
     void *batch = nullptr;        // root only: buffers of batched evaluations (plan.cpp)
     void *diag = nullptr;         // root only: diagonal-resolved trispectrum tables (plan.cpp)
     // root only: evaluate the spectrum box of another plan (fbs_plan_follow);

@@ -978,12 +978,18 @@ static void forward_or_follow(Plan &p, const float *field) {
     release_field(p, staged);
 }
 
-static void run_field(Plan &p, const float *field, bool quads) {
+// connected: the sums feed the connected trispectrum, a difference of nearly
+// equal numbers (an error of T grows up to 25 times in it), so they keep the
+// accumulation order of the tensor-memory contraction: both kernels' errors
+// against 64 bits are alike, but their roundings differ by more than the
+// 2e-5 within which a caller may rely on repeated results.
+static void run_field(Plan &p, const float *field, bool quads, bool connected = false) {
     const bool tc = p.precision != FBS_PREC_FP32;
     if (tc) FBS_CUDA(cudaMemsetAsync(p.d_errbuf, 0, sizeof(int), p.stream));
     forward_or_follow(p, field);
     for (Plan *lp : p.levels) {
         Plan &lv = *lp;
+        lv.gram_off = connected;
         lv.fused_active = quads && tc && tc_fused_usable(lv);
         zero_partials(lv, quads);
         launch_inverse_x(lv, false);
@@ -1128,6 +1134,7 @@ static void run_batch(Plan &p, const float *const *fields, int nf) {
         lv.slab = bl.slab;
         lv.nslabs = bl.nslabs;
         lv.fused_active = false;
+        lv.gram_off = false;
         try {
             const int M = lv.M, nb = lv.nbins;
             FBS_CUDA(cudaMemsetAsync(bl.tpart, 0, (size_t)nf * lv.part_blocks * std::max<size_t>(1, lv.ntri.size()) *
@@ -1570,10 +1577,12 @@ void fbs_plan_free(fbs_plan *plan) {
     if (plan->copy_stream) cudaStreamSynchronize(plan->copy_stream);
     cudaGetLastError();
     free_tc_state(*plan);
+    free_gram_state(*plan);
     free_batch(*plan);
     free_diag(*plan);
     for (Plan *lv : plan->levels) {
         free_tc_state(*lv);
+        free_gram_state(*lv);
         delete lv;
     }
     plan->levels.clear();
@@ -1890,7 +1899,7 @@ fbs_status fbs_trispectrum_connected(fbs_plan *plan, const float *field, double 
     }
     FBS_GUARD_BEGIN
     poll_device_errors(*plan);
-    run_field(*plan, field, true);
+    run_field(*plan, field, true, true);
     if (!plan->nquad.empty()) launch_connected(*plan, plan->d_Tc);
     bool host = false;
     copy_out(*plan, Tc, plan->d_Tc, plan->nquad.size(), host);
