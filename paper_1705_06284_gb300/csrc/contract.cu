@@ -2,127 +2,183 @@
 // Jeong_BI) on CUDA cores, the FP64 count sums that give the exact triangle
 // counts, and the FP64 normalisation epilogue (Eqs. Jeong_PS, Jeong_BI).
 //
-// Work is grouped by "outer pairs": for a bispectrum the pair (b, c) with
-// b <= c, carrying every a <= b that closes a triangle with it; the pair
-// product I_b I_c is formed once per point and reused for all its a.  For a
-// trispectrum the outer pair (c, d) carries inner pairs (a, b).
+// Work is grouped by "outer pairs": for a bispectrum one of a triplet's three
+// pairs, with the third bin as the inner row; for a trispectrum the pair
+// (c, d) with the product of the pair (a, b).  A pair's product is formed once
+// per point and reused for all its inner rows.
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <algorithm>
+#include <array>
+#include <map>
+#include <utility>
+#include <vector>
+
 #include "fbs_internal.h"
+#include "pair_cover.h"
 
 namespace fbs {
 
-static constexpr int kCThreads = 256;   // 8 warps
-static constexpr int kPtsPerLane = 16;  // 4 float4 per lane
-static constexpr int kChunk = 32 * kPtsPerLane;  // 512 points per chunk
+static constexpr int kCThreads = 512;     // 16 warps, one CTA per SM
+static constexpr int kGroupItems = 4096;  // items per CTA at most (12 bytes of shared memory each)
+
+__device__ __forceinline__ void lds_points(const float *row, int lane, int k, float2 &u, float2 &w) {
+    const float4 v = reinterpret_cast<const float4 *>(row)[lane + 32 * k];
+    u = make_float2(v.x, v.y);
+    w = make_float2(v.z, v.w);
+}
+
+// Stage I[b][q0 .. q0 + chunk) of every bin (asynchronous copies; the ragged
+// tail zero-padded by plain stores), one copy group.
+template <int chunk>
+__device__ __forceinline__ void stage_chunk(const float *I, long long bin_stride, long long npts, int nbins,
+                                            long long q0, float *dst) {
+    constexpr int n4 = chunk / 4;
+    for (int i = threadIdx.x; i < nbins * n4; i += kCThreads) {
+        const int b = i / n4, k = i % n4;
+        const long long q = q0 + 4LL * k;
+        const float *src = I + b * bin_stride + q;
+        if (q + 3 < npts) {
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(dst + 4 * i)),
+                         "l"(src)
+                         : "memory");
+        } else {
+            float4 v;
+            v.x = q + 0 < npts ? src[0] : 0.f;
+            v.y = q + 1 < npts ? src[1] : 0.f;
+            v.z = q + 2 < npts ? src[2] : 0.f;
+            v.w = 0.f;
+            reinterpret_cast<float4 *>(dst)[i] = v;
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
 
 // ------------------------------------------------------------------ FP32
-// grid.x: point-range blocks; grid.y: item groups (outer pairs [p0, p1)).
-// Each CTA sums over its point range; its FP64 totals are added to
-// part[blockIdx.x][item] (one row per CTA: no two CTAs touch the same word).
-template <bool QUAD>
-__global__ void __launch_bounds__(kCThreads) contract_fp32_kernel(
-    const float *__restrict__ I, long long bin_stride, long long npts, int nbins,
-    const int *__restrict__ pb, const int *__restrict__ pc, const int *__restrict__ pstart,
-    const int *__restrict__ ia, const int *__restrict__ ib, const int *__restrict__ iout,
-    const int *__restrict__ grp_pair0, int nitems_total, double *__restrict__ part, int chunk, int part_rows) {
+// grid.x: point-range blocks; grid.y: blocks of pair groups; grid.z: fields.
+// A warp holds the products of four outer pairs (one group) at PPL points per
+// lane and runs over the group's inner rows (single bins, or products of two
+// for quadruplets) two at a time: a row's values are loaded once and
+// multiplied into up to four items, and the lane sums of eight items are
+// reduced together (nine shuffles).  A chunk's FP32 sums go to shared memory,
+// one word per item, and are added to the FP64 totals by all threads: FP64
+// adds are scarce here (two a cycle per SM), and one lane's add per item, as
+// the one-pair form had it, costs as much as the products.  The next chunk's
+// fields are copied while this one's are used, and groups go to free warps,
+// the longest first.
+// What bounds it: shared-memory loads (69% of the cycles at 256^3, 32 linear
+// bins: 16 wavefronts per row and 16 per factor of a pair, for 512 points).
+// Measured against one pair at a time with one FP64 add per item: 256^3, 32
+// linear bins 4.89 -> 1.57 ms, 16 fields of 96^3, 24 bins 2.97 -> 0.96 ms,
+// 108^3, 10 log bins, triplets and quadruplets 460 -> 181 us.
+// bin_stride and the fields' base are multiples of 16 bytes (even grids).
+template <int PPL, bool QUAD>
+__global__ void __launch_bounds__(kCThreads, 1) contract_fp32_kernel(
+    const float *__restrict__ I, long long bin_stride, long long npts, int nbins, const FpGroup *__restrict__ groups,
+    const FpRow *__restrict__ rows, const int *__restrict__ iout, const int4 *__restrict__ blocks, int nitems_total,
+    double *__restrict__ part, int part_rows) {
+    constexpr int chunk = 32 * PPL;
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int g = blockIdx.y;
     // field blockIdx.z of a batch: its bins follow the previous fields' in I
     I += (long long)blockIdx.z * nbins * bin_stride;
-    const int p0 = grp_pair0[g], p1 = grp_pair0[g + 1];
-    const int it0 = pstart[p0], it1 = pstart[p1];
-    const int nloc = it1 - it0;
-    double *acc = reinterpret_cast<double *>(smraw);
-    float *sI = reinterpret_cast<float *>(smraw + (((size_t)nloc * sizeof(double) + 15) & ~(size_t)15));
-    for (int i = threadIdx.x; i < nloc; i += blockDim.x) acc[i] = 0.0;
+    const int4 blk = blocks[blockIdx.y];  // groups [x, y), first item z, items w
+    const int nloc = blk.w;
+    float *const sI = reinterpret_cast<float *>(smraw);  // two stages of nbins x chunk
+    double *const acc = reinterpret_cast<double *>(sI + 2 * nbins * chunk);
+    float *const tmp = reinterpret_cast<float *>(acc + nloc);
+    for (int i = threadIdx.x; i < nloc; i += kCThreads) acc[i] = 0.0;
 
     // contiguous point range of this CTA, in whole chunks
     const long long nchunks = (npts + chunk - 1) / chunk;
     const long long c0 = nchunks * blockIdx.x / gridDim.x;
     const long long c1 = nchunks * (blockIdx.x + 1) / gridDim.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nwarps = blockDim.x >> 5;
-    const int per_lane = chunk / 32;  // multiple of 4
+    const int lane = threadIdx.x & 31;
+    __shared__ int next_group;
+    if (threadIdx.x == 0) next_group = 0;
 
+    if (c0 < c1) stage_chunk<chunk>(I, bin_stride, npts, nbins, c0 * chunk, sI);
     for (long long ch = c0; ch < c1; ++ch) {
-        const long long q0 = ch * chunk;
-        const int nq = (int)min((long long)chunk, npts - q0);
-        __syncthreads();
-        // stage I[b][q0 .. q0+chunk) for every bin; zero-pad the ragged tail
-        const int n4 = chunk / 4;
-        for (int i = threadIdx.x; i < nbins * n4; i += blockDim.x) {
-            int b = i / n4, k = i - b * n4;
-            const long long q = q0 + 4LL * k;
-            float4 v;
-            if (q + 3 < npts && ((bin_stride & 3) == 0)) {
-                v = *reinterpret_cast<const float4 *>(I + b * bin_stride + q);
-            } else {
-                const float *src = I + b * bin_stride;
-                v.x = q + 0 < npts ? src[q + 0] : 0.f;
-                v.y = q + 1 < npts ? src[q + 1] : 0.f;
-                v.z = q + 2 < npts ? src[q + 2] : 0.f;
-                v.w = q + 3 < npts ? src[q + 3] : 0.f;
-            }
-            reinterpret_cast<float4 *>(sI + (size_t)b * chunk)[k] = v;
-        }
-        __syncthreads();
-        (void)nq;
-        for (int p = p0 + warp; p < p1; p += nwarps) {
-            const int b = pb[p], c = pc[p];
-            const float4 *rb = reinterpret_cast<const float4 *>(sI + (size_t)b * chunk);
-            const float4 *rc = reinterpret_cast<const float4 *>(sI + (size_t)c * chunk);
-            float pp[kPtsPerLane];
+        const float *const st = sI + ((ch - c0) & 1) * nbins * chunk;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();  // this chunk is staged; the other stage's readers and tmp's are done
+        if (ch + 1 < c1)
+            stage_chunk<chunk>(I, bin_stride, npts, nbins, (ch + 1) * chunk, sI + ((ch + 1 - c0) & 1) * nbins * chunk);
+        // groups, longest first, to the warps that are free
+        for (;;) {
+            int g = lane == 0 ? atomicAdd(&next_group, 1) : 0;
+            g = blk.x + __shfl_sync(0xffffffffu, g, 0);
+            if (g >= blk.y) break;
+            const FpGroup *G = groups + g;
+            float2 pp[4][PPL / 2];
+            const float *const rb = st + G->b[0] * chunk;
 #pragma unroll
-            for (int k = 0; k < kPtsPerLane / 4; ++k) {
-                if (4 * k < per_lane) {
-                    float4 u = rb[lane + 32 * k], w = rc[lane + 32 * k];
-                    pp[4 * k + 0] = u.x * w.x;
-                    pp[4 * k + 1] = u.y * w.y;
-                    pp[4 * k + 2] = u.z * w.z;
-                    pp[4 * k + 3] = u.w * w.w;
-                } else {
-                    pp[4 * k + 0] = pp[4 * k + 1] = pp[4 * k + 2] = pp[4 * k + 3] = 0.f;
+            for (int k = 0; k < PPL / 4; ++k) {
+                float2 u0, u1;
+                lds_points(rb, lane, k, u0, u1);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {  // pairs of a group mostly share their first bin
+                    float2 x0 = u0, x1 = u1, w0, w1;
+                    if (j > 0 && G->b[j] != G->b[0]) lds_points(st + G->b[j] * chunk, lane, k, x0, x1);
+                    lds_points(st + G->c[j] * chunk, lane, k, w0, w1);
+                    pp[j][2 * k] = __fmul2_rn(x0, w0);
+                    pp[j][2 * k + 1] = __fmul2_rn(x1, w1);
                 }
             }
-            const int e1 = pstart[p + 1];
-            for (int e = pstart[p]; e < e1; ++e) {
-                const float4 *ra = reinterpret_cast<const float4 *>(sI + (size_t)ia[e] * chunk);
-                float s = 0.f;
-                if (QUAD) {
-                    const float4 *rd = reinterpret_cast<const float4 *>(sI + (size_t)ib[e] * chunk);
+            const int4 *const rp = reinterpret_cast<const int4 *>(rows);
+            const int e1 = G->row1;
+            int4 n0 = rp[G->row0], n1 = rp[G->row0 + 1];
+            for (int e = G->row0; e < e1; e += 2) {  // a group has an even number of rows
+                const int4 r[2] = {n0, n1};
+                n0 = rp[min(e + 2, e1 - 2)];
+                n1 = rp[min(e + 3, e1 - 1)];
+                float s[2][4];
 #pragma unroll
-                    for (int k = 0; k < kPtsPerLane / 4; ++k) {
-                        if (4 * k < per_lane) {
-                            float4 u = ra[lane + 32 * k], w = rd[lane + 32 * k];
-                            s = fmaf(pp[4 * k + 0], u.x * w.x, s);
-                            s = fmaf(pp[4 * k + 1], u.y * w.y, s);
-                            s = fmaf(pp[4 * k + 2], u.z * w.z, s);
-                            s = fmaf(pp[4 * k + 3], u.w * w.w, s);
+                for (int h = 0; h < 2; ++h) {
+                    float2 v[PPL / 2];
+#pragma unroll
+                    for (int k = 0; k < PPL / 4; ++k) lds_points(st + r[h].x * chunk, lane, k, v[2 * k], v[2 * k + 1]);
+                    if (QUAD) {
+#pragma unroll
+                        for (int k = 0; k < PPL / 4; ++k) {
+                            float2 w0, w1;
+                            lds_points(st + r[h].y * chunk, lane, k, w0, w1);
+                            v[2 * k] = __fmul2_rn(v[2 * k], w0);
+                            v[2 * k + 1] = __fmul2_rn(v[2 * k + 1], w1);
                         }
                     }
-                } else {
 #pragma unroll
-                    for (int k = 0; k < kPtsPerLane / 4; ++k) {
-                        if (4 * k < per_lane) {
-                            float4 u = ra[lane + 32 * k];
-                            s = fmaf(pp[4 * k + 0], u.x, s);
-                            s = fmaf(pp[4 * k + 1], u.y, s);
-                            s = fmaf(pp[4 * k + 2], u.z, s);
-                            s = fmaf(pp[4 * k + 3], u.w, s);
-                        }
+                    for (int j = 0; j < 4; ++j) {  // items that do not exist are formed too: no branches
+                        float2 t = __fmul2_rn(pp[j][0], v[0]);
+#pragma unroll
+                        for (int k = 1; k < PPL / 2; ++k) t = __ffma2_rn(pp[j][k], v[k], t);
+                        s[h][j] = t.x + t.y;
                     }
                 }
+                // eight sums over 32 lanes: row (lane bit 4), pair (bits 3, 2)
+                const bool hi = lane & 16, p1 = lane & 8, p0 = lane & 4;
+                float a[4], b[2];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0) acc[e - it0] += (double)s;
+                for (int j = 0; j < 4; ++j)
+                    a[j] = (hi ? s[1][j] : s[0][j]) + __shfl_xor_sync(0xffffffffu, hi ? s[0][j] : s[1][j], 16);
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    b[j] = (p1 ? a[2 + j] : a[j]) + __shfl_xor_sync(0xffffffffu, p1 ? a[j] : a[2 + j], 8);
+                float t = (p0 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, p0 ? b[0] : b[1], 4);
+                t += __shfl_xor_sync(0xffffffffu, t, 2);
+                t += __shfl_xor_sync(0xffffffffu, t, 1);
+                const int mask = hi ? r[1].z : r[0].z, first = hi ? r[1].w : r[0].w, j = (lane >> 2) & 3;
+                if ((lane & 3) == 0 && (mask >> j & 1)) tmp[first + __popc(mask & ((1 << j) - 1))] = t;
             }
         }
+        __syncthreads();
+        if (threadIdx.x == 0) next_group = 0;  // read again past the next barrier
+        for (int i = threadIdx.x; i < nloc; i += kCThreads) acc[i] += (double)tmp[i];  // the same thread every time
     }
-    __syncthreads();
     double *row = part + ((long long)blockIdx.z * part_rows + blockIdx.x) * nitems_total;
-    for (int i = threadIdx.x; i < nloc; i += blockDim.x) row[iout[it0 + i]] += acc[i];
+    if (c0 < c1)
+        for (int i = threadIdx.x; i < nloc; i += kCThreads) row[iout[blk.z + i]] += acc[i];
 }
 
 // ------------------------------------------------------------------ reduce
@@ -364,52 +420,216 @@ static int num_sms() {
 
 int contract_blocks() { return 2 * num_sms(); }
 
-// item groups: consecutive outer pairs whose items fit in one CTA's smem accumulator
-std::vector<int> item_groups(const TaskList &t, int cap) {
-    std::vector<int> g{0};
-    int cur = 0;
-    for (int p = 0; p < t.npairs; ++p) {
-        int n = t.pstart[p + 1] - t.pstart[p];
-        if (cur > 0 && cur + n > cap) {
-            g.push_back(p);
-            cur = 0;
-        }
-        cur += n;
+// Groups of up to four outer pairs for the FP32 contraction, chosen so that
+// the pairs of a group share inner rows (each row's values are loaded once per
+// group): the next pair in order, then those of the following ones that add
+// the fewest rows.  Blocks of groups bound the items of a CTA.
+static void build_fp32_job(Plan &p, const TaskList &t, bool quads, FpJob &job) {
+    const int nb = p.nbins;
+    std::map<int, std::vector<std::pair<int, int>>> pairs;  // outer pair -> (inner row key, output)
+    if (quads) {
+        for (int i = 0; i < t.npairs; ++i)
+            for (int e = t.pstart[i]; e < t.pstart[i + 1]; ++e)
+                pairs[t.pb[i] * nb + t.pc[i]].push_back({t.ia[e] * nb + t.ib[e], t.iout[e]});
+    } else {
+        // each triplet by one of its three pairs: fewer pairs, more rows in common
+        std::vector<std::array<int, 3>> trip;
+        std::vector<int> out;
+        for (int i = 0; i < t.npairs; ++i)
+            for (int e = t.pstart[i]; e < t.pstart[i + 1]; ++e) {
+                std::array<int, 3> tr = {t.ia[e], t.pb[i], t.pc[i]};
+                std::sort(tr.begin(), tr.end());
+                trip.push_back(tr);
+                out.push_back(t.iout[e]);
+            }
+        const std::vector<int> key = cover_triplet_pairs(nb, trip);
+        for (size_t i = 0; i < trip.size(); ++i)
+            pairs[key[i]].push_back({trip[i][0] + trip[i][1] + trip[i][2] - key[i] / nb - key[i] % nb, out[i]});
     }
-    g.push_back(t.npairs);
-    return g;
+    std::vector<int> id;  // inner row keys -> bit
+    std::vector<int> bit_of((size_t)nb * nb, -1);
+    struct Outer {
+        int key;
+        std::vector<std::pair<int, int>> items;
+        std::vector<unsigned long long> bits;
+    };
+    std::vector<Outer> outer;
+    for (auto &kv : pairs) {
+        std::sort(kv.second.begin(), kv.second.end());
+        for (const auto &it : kv.second)
+            if (bit_of[it.first] < 0) {
+                bit_of[it.first] = (int)id.size();
+                id.push_back(it.first);
+            }
+    }
+    const size_t words = (id.size() + 63) / 64;
+    for (const auto &kv : pairs)
+        for (size_t i0 = 0; i0 < kv.second.size(); i0 += kGroupItems) {  // (a pair with more items: several times)
+            const size_t i1 = std::min(kv.second.size(), i0 + kGroupItems);
+            Outer o{kv.first, {kv.second.begin() + i0, kv.second.begin() + i1},
+                    std::vector<unsigned long long>(words, 0ULL)};
+            for (const auto &it : o.items) o.bits[bit_of[it.first] >> 6] |= 1ULL << (bit_of[it.first] & 63);
+            outer.push_back(std::move(o));
+        }
+    std::vector<FpGroup> groups;
+    std::vector<FpRow> rows;
+    std::vector<int> iout;
+    std::vector<int4> blocks;
+    std::vector<char> used(outer.size(), 0);
+    job.maxloc = 0;
+    int4 blk = make_int4(0, 0, 0, 0);
+    const auto close = [&] {
+        const int n = (int)groups.size() - blk.x;
+        if (n > 0) {
+            // two tasks per warp at least: groups split by rows (six at least, an
+            // even number) where there are fewer; the longest first
+            const int want = 2 * kCThreads / 32, parts = n >= want ? 1 : (want + n - 1) / n;
+            std::vector<FpGroup> tasks;
+            for (int i = blk.x; i < (int)groups.size(); ++i) {
+                FpGroup g = groups[i];
+                const int last = g.row1, len = std::max(6, ((last - g.row0 + parts - 1) / parts + 1) / 2 * 2);
+                while (g.row0 < last) {
+                    g.row1 = std::min(last, g.row0 + len);
+                    tasks.push_back(g);
+                    g.row0 = g.row1;
+                }
+            }
+            std::stable_sort(tasks.begin(), tasks.end(), [](const FpGroup &u, const FpGroup &v) {
+                return u.row1 - u.row0 > v.row1 - v.row0;
+            });
+            groups.resize(blk.x);
+            groups.insert(groups.end(), tasks.begin(), tasks.end());
+            blk.y = (int)groups.size();
+            job.maxloc = std::max(job.maxloc, blk.w);
+            blocks.push_back(blk);
+        }
+        blk = make_int4((int)groups.size(), 0, (int)iout.size(), 0);
+    };
+    for (size_t s = 0; s < outer.size(); ++s) {
+        if (used[s]) continue;
+        std::vector<int> pick{(int)s};
+        used[s] = 1;
+        std::vector<unsigned long long> bits = outer[s].bits;
+        size_t n = outer[s].items.size();
+        while (pick.size() < 4) {
+            int best = -1, score = -1000000, seen = 0;
+            for (size_t k = s + 1; k < outer.size() && seen < 48; ++k) {
+                if (used[k] || n + outer[k].items.size() > (size_t)kGroupItems) continue;
+                ++seen;
+                int both = 0;
+                for (size_t w = 0; w < words; ++w) both += __builtin_popcountll(bits[w] & outer[k].bits[w]);
+                const int sc = 2 * both - (int)outer[k].items.size();  // rows shared less rows added
+                if (sc > score) {
+                    score = sc;
+                    best = (int)k;
+                }
+            }
+            if (best < 0) break;
+            pick.push_back(best);
+            used[best] = 1;
+            n += outer[best].items.size();
+            for (size_t w = 0; w < words; ++w) bits[w] |= outer[best].bits[w];
+        }
+        if (blk.w > 0 && blk.w + n > (size_t)kGroupItems) close();
+        // the bin that most of the pairs have is their first factor, those pairs lead
+        int common = 0, most = 0;
+        for (int k : pick)
+            for (int bin : {outer[k].key / nb, outer[k].key % nb}) {
+                int cnt = 0;
+                for (int m : pick) cnt += outer[m].key / nb == bin || outer[m].key % nb == bin;
+                if (cnt > most) {
+                    most = cnt;
+                    common = bin;
+                }
+            }
+        const auto has = [&](int k) { return outer[k].key / nb == common || outer[k].key % nb == common; };
+        std::stable_partition(pick.begin(), pick.end(), has);
+        FpGroup g{};
+        for (int j = 0; j < 4; ++j) {  // empty places of a group repeat its first pair, without items
+            const int key = outer[pick[j < (int)pick.size() ? j : 0]].key;
+            const bool swap = key / nb != common && key % nb == common;
+            g.b[j] = swap ? key % nb : key / nb;
+            g.c[j] = swap ? key / nb : key % nb;
+        }
+        std::map<int, std::array<int, 4>> by_row;  // inner row -> outputs of the four pairs (-1: none)
+        for (size_t j = 0; j < pick.size(); ++j)
+            for (const auto &it : outer[pick[j]].items) {
+                auto at = by_row.emplace(it.first, std::array<int, 4>{-1, -1, -1, -1});
+                at.first->second[j] = it.second;
+            }
+        g.row0 = (int)rows.size();
+        for (const auto &kv : by_row) {
+            FpRow r{};
+            r.x = quads ? kv.first / nb : kv.first;
+            r.y = quads ? kv.first % nb : 0;
+            r.first = blk.w;
+            for (int j = 0; j < 4; ++j)
+                if (kv.second[j] >= 0) {
+                    r.mask |= 1 << j;
+                    iout.push_back(kv.second[j]);
+                    ++blk.w;
+                }
+            rows.push_back(r);
+        }
+        if ((rows.size() - g.row0) % 2) rows.push_back(FpRow{});  // no items
+        g.row1 = (int)rows.size();
+        groups.push_back(g);
+    }
+    close();
+    const auto up = [&](const void *v, size_t bytes) {
+        void *d = p.dalloc(std::max<size_t>(bytes, 16));
+        FBS_CUDA(cudaMemcpyAsync(d, v, bytes, cudaMemcpyHostToDevice, p.stream));
+        return d;
+    };
+    job.d_groups = (FpGroup *)up(groups.data(), groups.size() * sizeof(FpGroup));
+    job.d_rows = (FpRow *)up(rows.data(), rows.size() * sizeof(FpRow));
+    job.d_iout = (int *)up(iout.data(), iout.size() * sizeof(int));
+    job.d_blocks = (int4 *)up(blocks.data(), blocks.size() * sizeof(int4));
+    FBS_CUDA(cudaStreamSynchronize(p.stream));  // host tables go out of scope
+    job.nblocks = (int)blocks.size();
+    job.built = true;
+}
+
+// Tables of a level's FP32 contraction, built when the plan first has a use for
+// them (its creation or a change of precision, never inside an evaluation that
+// a caller may be capturing).
+void prepare_fp32(Plan &p, bool trip, bool quads) {
+    if (trip && !p.fpt.built && p.ttask.nitems > 0) build_fp32_job(p, p.ttask, false, p.fpt);
+    if (quads && !p.fpq.built && p.qtask.nitems > 0) build_fp32_job(p, p.qtask, true, p.fpq);
 }
 
 void launch_contract_fp32(Plan &p, const float *islab, long long npts, long long slab_stride,
                           bool quads, int nf, double *part_batch) {
     const TaskList &t = quads ? p.qtask : p.ttask;
     if (t.nitems == 0) return;
-    const std::vector<int> &grp = quads ? p.qgrp : p.tgrp;
-    const int *d_grp = quads ? p.d_qgrp : p.d_tgrp;
-    const int ngrp = (int)grp.size() - 1;
-    int maxloc = 0;
-    for (int g = 0; g < ngrp; ++g)
-        maxloc = std::max(maxloc, t.pstart[grp[g + 1]] - t.pstart[grp[g]]);
-    int chunk = kChunk;
-    // shrink the staged chunk for many bins (smem budget ~200 KB)
-    while (chunk > 128 && (size_t)p.nbins * chunk * 4 + (size_t)maxloc * 8 > 200 * 1024) chunk /= 2;
-    const size_t sm = (((size_t)maxloc * 8 + 15) & ~(size_t)15) + (size_t)p.nbins * chunk * 4;
+    prepare_fp32(p, !quads, quads);
+    const FpJob &job = quads ? p.fpq : p.fpt;
+    // 512 points per chunk; fewer where that leaves SMs without a chunk or two
+    // stages do not fit
+    int ppl = 16;
+    const auto smem = [&] { return (size_t)job.maxloc * 12 + 16 + (size_t)p.nbins * 256 * ppl; };
+    while (ppl > 4 && (smem() > 220 * 1024 || npts * nf < 32LL * ppl * num_sms())) ppl /= 2;
+    const size_t sm = smem();
     KTimer tm(p, quads ? KC_QUAD : KC_CONTRACT);
-    dim3 grid(std::max(1, p.part_blocks / nf), ngrp, nf);
+    // one CTA per SM over the fields and blocks, or two rounds of them where one
+    // would leave more than 3% of the SMs idle
+    const int per = nf * job.nblocks, one = num_sms() / per;
+    const int G = (num_sms() - one * per) * 33 > num_sms() ? std::max(1, 2 * num_sms() / per) : one;
+    dim3 grid(std::min(G, p.part_blocks), job.nblocks, nf);
+    const auto run = [&](auto k) {
+        FBS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        k<<<grid, kCThreads, sm, p.stream>>>(islab, slab_stride, npts, p.nbins, job.d_groups, job.d_rows, job.d_iout,
+                                             job.d_blocks, t.nitems,
+                                             part_batch ? part_batch : quads ? p.d_qpart : p.d_tpart, p.part_blocks);
+    };
     if (quads) {
-        auto k = contract_fp32_kernel<true>;
-        FBS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        k<<<grid, kCThreads, sm, p.stream>>>(islab, slab_stride, npts, p.nbins, p.d_qpb, p.d_qpc,
-                                             p.d_qps, p.d_qia, p.d_qib, p.d_qout, d_grp,
-                                             t.nitems, part_batch ? part_batch : p.d_qpart, chunk,
-                                             p.part_blocks);
+        if (ppl == 16) run(contract_fp32_kernel<16, true>);
+        else if (ppl == 8) run(contract_fp32_kernel<8, true>);
+        else run(contract_fp32_kernel<4, true>);
     } else {
-        auto k = contract_fp32_kernel<false>;
-        FBS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        k<<<grid, kCThreads, sm, p.stream>>>(islab, slab_stride, npts, p.nbins, p.d_tpb, p.d_tpc,
-                                             p.d_tps, p.d_tia, nullptr, p.d_tout, d_grp,
-                                             t.nitems, part_batch ? part_batch : p.d_tpart, chunk,
-                                             p.part_blocks);
+        if (ppl == 16) run(contract_fp32_kernel<16, false>);
+        else if (ppl == 8) run(contract_fp32_kernel<8, false>);
+        else run(contract_fp32_kernel<4, false>);
     }
     FBS_CUDA(cudaGetLastError());
 }

@@ -72,6 +72,25 @@ struct TaskList {
     std::vector<int> ia, ib, iout;          // inner item bins (ib = -1 for triplets), output index
 };
 
+// FP32 contraction: groups of four outer pairs (products of bins b and c) with
+// the inner rows they meet (bin x, or the product of x and y); mask: which of
+// the four have an item with the row, `first` the first of them among the
+// block's items.
+struct FpGroup {
+    int b[4], c[4], row0, row1;
+};
+struct alignas(16) FpRow {
+    int x, y, mask, first;
+};
+struct FpJob {
+    FpGroup *d_groups = nullptr;
+    FpRow *d_rows = nullptr;
+    int *d_iout = nullptr;    // block's item -> output
+    int4 *d_blocks = nullptr; // groups [x, y), first item, items
+    int nblocks = 0, maxloc = 0;
+    bool built = false;
+};
+
 // ---------------------------------------------------------------- timing
 enum KernelClass {
     KC_FWD_Z = 0,
@@ -157,7 +176,7 @@ void launch_normalise_batch(Plan &root, bool quads, int nf, const double *tnum, 
 void launch_connected(Plan &root, double *d_Tc);
 std::vector<int> fast_grids();  // grids with compile-time-radix kernels for every inverse stage
 void zero_partials(Plan &p, bool quads);
-std::vector<int> item_groups(const TaskList &t, int cap);
+void prepare_fp32(Plan &level, bool trip, bool quads);
 int contract_blocks();
 
 // ---------------------------------------------------------------- plan
@@ -221,8 +240,7 @@ struct Plan {
     std::vector<double> nquad;   // FP64 ordered quadruple counts (the nearest double of nquad128)
     std::vector<U128> nquad128;  // exact ordered quadruple counts (root plan, output order)
     TaskList ttask, qtask;
-    std::vector<int> tgrp, qgrp;  // item groups of the FP32 contraction (outer-pair ranges)
-    int *d_tgrp = nullptr, *d_qgrp = nullptr;
+    FpJob fpt, fpq;              // FP32 contraction of the triplets, of the quadruplets
 
     long long A_elems = 0;       // complex elements of the x-stage output (all bins)
     long long G_plane = 0;       // complex elements of the y-stage output per plane (all bins)
@@ -253,10 +271,6 @@ struct Plan {
     BinGeom *d_geom = nullptr;
     float2 *d_tw = nullptr;      // e^{-2 pi i k/N}, k < N (FP32)
     double2 *d_tw64 = nullptr;   // e^{-2 pi i k/M}, k < M, in FP64 (count fields)
-    // task lists on device
-    int *d_tpb = nullptr, *d_tpc = nullptr, *d_tps = nullptr, *d_tia = nullptr, *d_tout = nullptr;
-    int *d_qpb = nullptr, *d_qpc = nullptr, *d_qps = nullptr, *d_qia = nullptr, *d_qib = nullptr,
-        *d_qout = nullptr;
     // accumulators
     int part_blocks = 0;          // number of FP64 partial rows
     double *d_tpart = nullptr;    // [part_blocks][ntrip]

@@ -824,8 +824,6 @@ static void create_plan(Plan &p, const double *edges, const void *blob = nullptr
     for (size_t l = 0; l < grids.size(); ++l) {
         Plan &lv = *p.levels[l];
         build_tasks(lv);
-        lv.tgrp = item_groups(lv.ttask, 8192);
-        lv.qgrp = item_groups(lv.qtask, 8192);
         const int M = lv.M, lnb = lv.nbins;
         const long long per_plane = (long long)lnb * M * M * 4 + lv.G_plane * 8;
         const long long budget = slab_budget_bytes();
@@ -854,19 +852,8 @@ static void create_plan(Plan &p, const double *edges, const void *blob = nullptr
         lv.d_G = sG;
         lv.d_I = sI;
         lv.d_geom = upload(lv, lv.geom);
-        lv.d_tpb = upload(lv, lv.ttask.pb);
-        lv.d_tpc = upload(lv, lv.ttask.pc);
-        lv.d_tps = upload(lv, lv.ttask.pstart);
-        lv.d_tia = upload(lv, lv.ttask.ia);
-        lv.d_tout = upload(lv, lv.ttask.iout);
-        lv.d_tgrp = upload(lv, lv.tgrp);
-        lv.d_qpb = upload(lv, lv.qtask.pb);
-        lv.d_qpc = upload(lv, lv.qtask.pc);
-        lv.d_qps = upload(lv, lv.qtask.pstart);
-        lv.d_qia = upload(lv, lv.qtask.ia);
-        lv.d_qib = upload(lv, lv.qtask.ib);
-        lv.d_qout = upload(lv, lv.qtask.iout);
-        lv.d_qgrp = upload(lv, lv.qgrp);
+        // quadruplets the tensor cores cannot hold run in FP32 in every precision
+        prepare_fp32(lv, p.precision == FBS_PREC_FP32, quads_on);
         lv.d_gtrip = upload(lv, lv.gtrip);
         lv.d_gquad = upload(lv, lv.gquad);
         lv.d_pbin = upload(lv, lv.pbin);
@@ -1634,9 +1621,13 @@ fbs_status fbs_plan_set_precision(fbs_plan *plan, int precision) {
         set_error("bad plan or precision");
         return FBS_ERR_ARG;
     }
+    FBS_GUARD_BEGIN
+    if (precision == FBS_PREC_FP32)
+        for (Plan *lv : plan->levels) prepare_fp32(*lv, true, false);
     plan->precision = precision;
     for (Plan *lv : plan->levels) lv->precision = precision;
     return FBS_OK;
+    FBS_GUARD_END
 }
 
 static bool set_plan_option(Plan *plan, int option, int value);
