@@ -78,7 +78,7 @@ template <int PPL, bool QUAD>
 __global__ void __launch_bounds__(kCThreads, 1) contract_fp32_kernel(
     const float *__restrict__ I, long long bin_stride, long long npts, int nbins, const FpGroup *__restrict__ groups,
     const FpRow *__restrict__ rows, const int *__restrict__ iout, const int4 *__restrict__ blocks, int nitems_total,
-    double *__restrict__ part, int part_rows) {
+    double *__restrict__ part, int part_rows, int first) {
     constexpr int chunk = 32 * PPL;
     extern __shared__ __align__(16) unsigned char smraw[];
     // field blockIdx.z of a batch: its bins follow the previous fields' in I
@@ -177,47 +177,74 @@ __global__ void __launch_bounds__(kCThreads, 1) contract_fp32_kernel(
         for (int i = threadIdx.x; i < nloc; i += kCThreads) acc[i] += (double)tmp[i];  // the same thread every time
     }
     double *row = part + ((long long)blockIdx.z * part_rows + blockIdx.x) * nitems_total;
-    if (c0 < c1)
-        for (int i = threadIdx.x; i < nloc; i += kCThreads) row[iout[blk.z + i]] += acc[i];
+    for (int i = threadIdx.x; i < nloc; i += kCThreads) {
+        double &d = row[iout[blk.z + i]];
+        d = first ? acc[i] : d + acc[i];
+    }
 }
 
 // ------------------------------------------------------------------ reduce
-// out[map[i]] = scale * sum_r part[r*ld + i], i < n (rows summed in a fixed
-// order, deterministic); map == nullptr: out[i].
-// Field blockIdx.y of a batch: its partials at part + y*sfs, its outputs at out + y*ofs.
-__global__ void reduce_rows_kernel(const double *__restrict__ part, int rows, int n, int ld,
-                                   double *__restrict__ out, double scale, const int *__restrict__ map,
-                                   long long sfs, long long ofs) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    part += blockIdx.y * sfs;
-    out += blockIdx.y * ofs;
-    double s = 0.0;
-    for (int r = 0; r < rows; ++r) s += part[(long long)r * ld + i];
-    out[map ? map[i] : i] = scale * s;
-}
+// Sums of a level's partials, one launch: blocks [0, nblk[0]) and [nblk[0],
+// nblk[0] + nblk[1]) take 32 items each of the two segments, out[map[i]] =
+// scale * sum_r part[r * ld + i] over the rows the contraction wrote; the rest
+// take one bin each, sumsq[pbin[b]] = scale * sum_r sq[b][r].  Eight threads
+// share an item's rows (one thread per item and 304 rows, most of them zero,
+// took 40 to 50 us of dependent loads for any size).  Every sum has a fixed
+// order.  Field blockIdx.y of a batch: partials sfs, outputs ofs further on.
+struct ReduceSeg {
+    const double *part;
+    const int *map;
+    double *out;
+    int n, ld, rows;
+    long long sfs, ofs;
+};
+struct ReduceArgs {
+    ReduceSeg seg[2];
+    int nblk[2];
+    const double *sq;
+    const int *pbin;
+    double *sumsq;
+    int sqrows;
+    long long sfs, ofs;
+    double scale;
+};
 
-// out[map[j]] = scale * sum_r part[j][r] for every j with map[j] >= 0: one
-// block per j, strided partial sums then a fixed-shape tree (deterministic
-// for a given launch shape).
-__global__ void __launch_bounds__(256) reduce_cols_kernel(const double *__restrict__ part, int rows,
-                                                          double *__restrict__ out, double scale,
-                                                          const int *__restrict__ map, long long sfs,
-                                                          long long ofs) {
+__global__ void __launch_bounds__(256) level_reduce_kernel(const __grid_constant__ ReduceArgs a) {
     __shared__ double red[256];
-    const int j = blockIdx.x;
-    if (map[j] < 0) return;
-    part += blockIdx.y * sfs;  // field blockIdx.y of a batch
-    out += blockIdx.y * ofs;
+    const int tid = threadIdx.x;
+    int blk = blockIdx.x;
+    const int which = blk < a.nblk[0] ? 0 : blk < a.nblk[0] + a.nblk[1] ? 1 : 2;
+    if (which < 2) {
+        const ReduceSeg &g = a.seg[which];
+        if (which) blk -= a.nblk[0];
+        const int i = 32 * blk + (tid & 31), ty = tid >> 5;
+        const double *part = g.part + blockIdx.y * g.sfs;
+        double s = 0.0;
+        if (i < g.n) {
+#pragma unroll 4
+            for (int r = ty; r < g.rows; r += 8) s += part[(long long)r * g.ld + i];
+        }
+        red[tid] = s;
+        __syncthreads();
+        if (ty == 0 && i < g.n) {
+            for (int k = 1; k < 8; ++k) s += red[tid + 32 * k];
+            g.out[blockIdx.y * g.ofs + (g.map ? g.map[i] : i)] = a.scale * s;
+        }
+        return;
+    }
+    blk -= a.nblk[0] + a.nblk[1];
+    if (a.pbin[blk] < 0) return;
+    const double *sq = a.sq + blockIdx.y * a.sfs + (long long)blk * a.sqrows;
     double s = 0.0;
-    for (int r = threadIdx.x; r < rows; r += blockDim.x) s += part[(long long)j * rows + r];
-    red[threadIdx.x] = s;
+#pragma unroll 4
+    for (int r = tid; r < a.sqrows; r += 256) s += sq[r];
+    red[tid] = s;
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+    for (int w = 128; w > 0; w >>= 1) {
+        if (tid < w) red[tid] += red[tid + w];
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[map[j]] = scale * red[0];
+    if (tid == 0) a.sumsq[blockIdx.y * a.ofs + a.pbin[blk]] = a.scale * red[0];
 }
 
 // ------------------------------------------------------------------ normalise
@@ -620,8 +647,10 @@ void launch_contract_fp32(Plan &p, const float *islab, long long npts, long long
         FBS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
         k<<<grid, kCThreads, sm, p.stream>>>(islab, slab_stride, npts, p.nbins, job.d_groups, job.d_rows, job.d_iout,
                                              job.d_blocks, t.nitems,
-                                             part_batch ? part_batch : quads ? p.d_qpart : p.d_tpart, p.part_blocks);
+                                             part_batch ? part_batch : quads ? p.d_qpart : p.d_tpart, p.part_blocks,
+                                             p.first_slab);
     };
+    (quads ? p.qrows : p.trows) = (int)grid.x;
     if (quads) {
         if (ppl == 16) run(contract_fp32_kernel<16, true>);
         else if (ppl == 8) run(contract_fp32_kernel<8, true>);
@@ -632,23 +661,6 @@ void launch_contract_fp32(Plan &p, const float *islab, long long npts, long long
         else run(contract_fp32_kernel<4, false>);
     }
     FBS_CUDA(cudaGetLastError());
-}
-
-void zero_partials(Plan &p, bool quads) {
-    if (p.fused_active) {
-        FBS_CUDA(cudaMemsetAsync(p.d_fpart, 0,
-                                 (size_t)p.part_blocks * (p.ttask.nitems + p.qtask.nitems) * sizeof(double),
-                                 p.stream));
-    } else {
-        if (p.d_tpart && p.ttask.nitems > 0)
-            FBS_CUDA(cudaMemsetAsync(p.d_tpart, 0, (size_t)p.part_blocks * p.ttask.nitems * sizeof(double),
-                                     p.stream));
-        if (quads && p.d_qpart && p.qtask.nitems > 0)
-            FBS_CUDA(cudaMemsetAsync(p.d_qpart, 0, (size_t)p.part_blocks * p.qtask.nitems * sizeof(double),
-                                     p.stream));
-    }
-    FBS_CUDA(cudaMemsetAsync(p.d_sumsq_part, 0,
-                             (size_t)p.nbins * p.M * zstage_row_groups(p.M) * sizeof(double), p.stream));
 }
 
 // A level's sums over its M^3 grid -> sums over the N^3 grid ((N/M)^3), into
@@ -667,27 +679,23 @@ void launch_level_reduce_batch(Plan &p, bool quads, int nf, const double *tpart,
     Plan &R = p.root();
     KTimer tm(p, KC_REDUCE);
     const double r = (double)R.N / (double)p.M;
-    const double scale = r * r * r;
-    const int rows = p.M * zstage_row_groups(p.M);
-    int n = p.ttask.nitems;
-    if (n > 0) {
-        const int ld = p.fused_active ? n + p.qtask.nitems : n;
-        dim3 grid((n + 255) / 256, nf);
-        reduce_rows_kernel<<<grid, 256, 0, p.stream>>>(tpart, p.part_blocks, n, ld, tnum, scale, p.d_gtrip,
-                                                       (long long)p.part_blocks * ld, (long long)R.ntri.size());
-        FBS_CUDA(cudaGetLastError());
-    }
-    if (quads && p.qtask.nitems > 0) {
-        int m = p.qtask.nitems;
-        const double *src = p.fused_active ? p.d_fpart + p.ttask.nitems : p.d_qpart;
-        const int ld = p.fused_active ? m + p.ttask.nitems : m;
-        reduce_rows_kernel<<<(m + 255) / 256, 256, 0, p.stream>>>(src, p.part_blocks, m, ld, R.d_qnum, scale,
-                                                                  p.d_gquad, 0, 0);
-        FBS_CUDA(cudaGetLastError());
-    }
-    dim3 gc(p.nbins, nf);
-    reduce_cols_kernel<<<gc, 256, 0, p.stream>>>(sq, rows, sumsq, scale, p.d_pbin, (long long)p.nbins * rows,
-                                                 (long long)R.nbins);
+    ReduceArgs a{};
+    a.scale = r * r * r;
+    const int n = p.ttask.nitems, m = quads ? p.qtask.nitems : 0;
+    const int ld = p.fused_active ? n + m : n;
+    a.seg[0] = ReduceSeg{tpart, p.d_gtrip, tnum, n, ld, p.trows, (long long)p.part_blocks * ld,
+                         (long long)R.ntri.size()};
+    a.nblk[0] = (n + 31) / 32;
+    if (p.fused_active) a.seg[1] = ReduceSeg{p.d_fpart + n, p.d_gquad, R.d_qnum, m, ld, p.trows, 0, 0};
+    else a.seg[1] = ReduceSeg{p.d_qpart, p.d_gquad, R.d_qnum, m, m, p.qrows, 0, 0};
+    a.nblk[1] = (m + 31) / 32;
+    a.sq = sq;
+    a.pbin = p.d_pbin;
+    a.sumsq = sumsq;
+    a.sqrows = p.M * zstage_row_groups(p.M);
+    a.sfs = (long long)p.nbins * a.sqrows;
+    a.ofs = R.nbins;
+    level_reduce_kernel<<<dim3(a.nblk[0] + a.nblk[1] + p.nbins, nf), 256, 0, p.stream>>>(a);
     FBS_CUDA(cudaGetLastError());
 }
 
@@ -734,8 +742,11 @@ void launch_count_contraction(Plan &p, const double *noct, int nbins_all, int, c
     dim3 g(blocks, ngrp);
     count_kernel<<<g, 256, sm, p.stream>>>(noct, nbins_all, H, d_items, arity, nitems, grp, part, kCntChunk);
     FBS_CUDA(cudaGetLastError());
-    reduce_rows_kernel<<<(nitems + 255) / 256, 256, 0, p.stream>>>(part, blocks, nitems, nitems, d_den, 1.0,
-                                                                   nullptr, 0, 0);
+    ReduceArgs a{};
+    a.scale = 1.0;
+    a.seg[0] = ReduceSeg{part, nullptr, d_den, nitems, nitems, blocks, 0, 0};
+    a.nblk[0] = (nitems + 31) / 32;
+    level_reduce_kernel<<<a.nblk[0], 256, 0, p.stream>>>(a);
     FBS_CUDA(cudaGetLastError());
 }
 

@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
     contract_gram_kernel(const __grid_constant__ CUtensorMap fmap, long long npts, int nbins,
                          const GramGroup *__restrict__ groups, const GramTable *__restrict__ tables,
                          const __grid_constant__ GramUnits<CAP> units, const int *__restrict__ iout, int nitems_total, double *__restrict__ part, int part_rows,
-                         int F, int S, int lanes, int stage_atoms, int lolo, int *__restrict__ err, long long wait_limit) {
+                         int F, int S, int lanes, int stage_atoms, int lolo, int first, int *__restrict__ err, long long wait_limit) {
     extern __shared__ __align__(1024) unsigned char smraw[];
     __shared__ GramBars bars;
     __shared__ uint32_t tmem_slot;
@@ -472,7 +472,11 @@ __global__ void __launch_bounds__(kGThreads, 1)
     if (warp == kMma)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
     double *row = part + ((long long)blockIdx.z * part_rows + blockIdx.x) * nitems_total;
-    for (int i = tid; i < g.nitems; i += kGThreads) row[iout[g.item0 + i]] += (double)sums[i].x - (double)sums[i].y;
+    for (int i = tid; i < g.nitems; i += kGThreads) {
+        const double v = (double)sums[i].x - (double)sums[i].y;
+        double &d = row[iout[g.item0 + i]];
+        d = first ? v : d + v;
+    }
 }
 
 }  // namespace
@@ -725,6 +729,7 @@ void launch_gram(Plan &p, bool fused, const float *islab, long long npts, long l
     const size_t sm = std::max<size_t>(gram_smem(p, job, F, S), 116 * 1024);  // one CTA per SM
     const CUtensorMap fmap = field_map(islab, npts, slab_stride, p.nbins, nf * p.nbins, kPts, false);
     KTimer tm(p, kclass);
+    p.trows = G;
     job.last_F = F;
     job.last_S = S;
     const auto run = [&](auto kernel, auto units) {
@@ -732,7 +737,7 @@ void launch_gram(Plan &p, bool fused, const float *islab, long long npts, long l
         FBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
         kernel<<<dim3(G, job.ngroups, nf), kGThreads, sm, p.stream>>>(
             fmap, npts, p.nbins, job.d_groups, job.d_tables, units, job.d_iout, nitems_total, part, p.part_blocks, F,
-            S, lanes, job.maxatoms, fused ? 0 : 1, p.root().d_errbuf, p.tc_wait_limit > 0 ? p.tc_wait_limit : kWaitCycles);
+            S, lanes, job.maxatoms, fused ? 0 : 1, p.first_slab, p.root().d_errbuf, p.tc_wait_limit > 0 ? p.tc_wait_limit : kWaitCycles);
     };
     // the argument block sized for the job (1.7, 3.5 or 11.5 KB)
     const bool fixed = job.maxunits <= kProd;

@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                        const int *__restrict__ grp_tile0, const int *__restrict__ iout,
                        int nitems_total, double *__restrict__ part, int x3, int flush_every,
                        int *__restrict__ err, long long wait_limit, int part_rows, int merged, int nsb,
-                       const int *__restrict__ ifeed, int nbuild, int stacked_arg) {
+                       const int *__restrict__ ifeed, int nbuild, int stacked_arg, int first) {
     static_assert(AW == 16 || AW == 8, "A-operand warps: 16 or 8");
     static_assert(!FEED || AW == 16, "inner pair rows from operand A: the A warps build operand B");
     static_assert(KA == 1 || KA == 2, "K-atoms per chunk: 1 or 2");
@@ -755,9 +755,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     if (warp == kMmaWarp)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
     double *row = part + ((long long)blockIdx.z * part_rows + blockIdx.x) * nitems_total;
-    for (int i = tid; i < nloc; i += kTcThreads)
-        row[iout[it0 + i]] += ((double)acc[i].x - (double)acc[i].y) +
-                              (stacked ? (double)acc2[i].x - (double)acc2[i].y : 0.0);
+    for (int i = tid; i < nloc; i += kTcThreads) {
+        const double v = ((double)acc[i].x - (double)acc[i].y) +
+                         (stacked ? (double)acc2[i].x - (double)acc2[i].y : 0.0);
+        double &d = row[iout[it0 + i]];
+        d = first ? v : d + v;
+    }
 }
 
 
@@ -1450,12 +1453,16 @@ static bool launch_wide(Plan &p, const float *islab, long long npts, long long s
     if (G > p.part_blocks) G = p.part_blocks;
     const size_t sm = std::max<size_t>(wide_smem_bytes(p.nbins, w.maxloc), 116 * 1024);
     const TaskList &t = quads ? p.qtask : p.ttask;
+    // this kernel adds to its partial rows: they start at zero
+    double *const part = quads ? p.d_qpart : p.d_tpart;
+    (quads ? p.qrows : p.trows) = G;
+    if (p.first_slab) FBS_CUDA(cudaMemsetAsync(part, 0, (size_t)G * t.nitems * sizeof(double), p.stream));
     KTimer tm(p, quads ? KC_QUAD_TC : KC_CONTRACT_TC);
     FBS_CUDA(cudaFuncSetAttribute(contract_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     dim3 grid(G, ngrp);
     contract_wide_kernel<<<grid, kWideThreads, sm, p.stream>>>(
         islab, slab_stride, npts, p.nbins, w.nleft, w.d_left, w.d_rights, w.nright, w.d_item_out, t.nitems,
-        quads ? p.d_qpart : p.d_tpart, p.precision == FBS_PREC_BF16 ? 0 : 1, 16, st.d_err, tc_wait_limit(p));
+        part, p.precision == FBS_PREC_BF16 ? 0 : 1, 16, st.d_err, tc_wait_limit(p));
     FBS_CUDA(cudaGetLastError());
     return true;
 }
@@ -1564,6 +1571,7 @@ static void launch_job(Plan &p, TcJob &job, const float *islab, long long npts, 
     const CUtensorMap fmap = field_map(islab, npts, slab_stride, p.nbins, nf * p.nbins, 32, true);
     KTimer tm(p, kclass);
     dim3 grid(G, ngrp, nf);
+    (kclass == KC_QUAD_TC && !p.fused_active ? p.qrows : p.trows) = G;
     job.last_merged = stacked ? 2 : merged;
     job.last_ka = ka;
     job.last_nsb = nsb;
@@ -1579,7 +1587,7 @@ static void launch_job(Plan &p, TcJob &job, const float *islab, long long npts, 
         contract_tc_kernel<A, S, W, K, F><<<grid, kTcThreads, sm, p.stream>>>(                          \
             fmap, npts, p.nbins, job.Npad, tstr, job.ninner, job.d_inner, job.d_pairs, job.npairs,      \
             job.d_grp, job.d_iout, nitems_total, part, x3, flush_every, st.d_err, tc_wait_limit(p),     \
-            p.part_blocks, merged, nsb, ifeed, nbuild, stacked);                                      \
+            p.part_blocks, merged, nsb, ifeed, nbuild, stacked, p.first_slab);                                      \
     }
     bool launched = false;
     FBS_TC_LAUNCH(2, 2, 16, 1, false)

@@ -175,7 +175,6 @@ void launch_normalise_batch(Plan &root, bool quads, int nf, const double *tnum, 
 // Connected trispectrum of the last evaluation into d_Tc[nquad] (root).
 void launch_connected(Plan &root, double *d_Tc);
 std::vector<int> fast_grids();  // grids with compile-time-radix kernels for every inverse stage
-void zero_partials(Plan &p, bool quads);
 void prepare_fp32(Plan &level, bool trip, bool quads);
 int contract_blocks();
 
@@ -273,6 +272,8 @@ struct Plan {
     double2 *d_tw64 = nullptr;   // e^{-2 pi i k/M}, k < M, in FP64 (count fields)
     // accumulators
     int part_blocks = 0;          // number of FP64 partial rows
+    int trows = 0, qrows = 0;     // rows this evaluation's contractions write (triplets or fused, quadruplets)
+    int first_slab = 1;           // the contraction stores its partial rows (later slabs add to them)
     double *d_tpart = nullptr;    // [part_blocks][ntrip]
     double *d_qpart = nullptr;    // [part_blocks][nquad]
     double *d_fpart = nullptr;    // [part_blocks][ntrip + nquad] of the fused tensor-core pass

@@ -978,7 +978,6 @@ static void run_field(Plan &p, const float *field, bool quads, bool connected = 
         Plan &lv = *lp;
         lv.gram_off = connected;
         lv.fused_active = quads && tc && tc_fused_usable(lv);
-        zero_partials(lv, quads);
         launch_inverse_x(lv, false);
         const int M = lv.M;
         const long long plane = (long long)M * M;
@@ -986,6 +985,7 @@ static void run_field(Plan &p, const float *field, bool quads, bool connected = 
             const int x0 = s * lv.slab;
             const int nx = std::min(lv.slab, M - x0);
             if (nx <= 0) break;
+            lv.first_slab = s == 0;
             launch_inverse_yz_slab(lv, x0, nx, lv.d_I);
             const long long npts = (long long)nx * plane;
             const long long stride = (long long)lv.slab * plane;
@@ -1124,16 +1124,13 @@ static void run_batch(Plan &p, const float *const *fields, int nf) {
         lv.gram_off = false;
         try {
             const int M = lv.M, nb = lv.nbins;
-            FBS_CUDA(cudaMemsetAsync(bl.tpart, 0, (size_t)nf * lv.part_blocks * std::max<size_t>(1, lv.ntri.size()) *
-                                                      sizeof(double), p.stream));
-            FBS_CUDA(cudaMemsetAsync(bl.sq, 0, (size_t)nf * nb * M * zstage_row_groups(M) * sizeof(double),
-                                     p.stream));
             launch_inverse_x_geom(lv, bl.d_vgeom, nb, nf * nb);
             const long long plane = (long long)M * M;
             for (int s = 0; s < bl.nslabs; ++s) {
                 const int x0 = s * bl.slab;
                 const int nx = std::min(bl.slab, M - x0);
                 if (nx <= 0) break;
+                lv.first_slab = s == 0;
                 launch_inverse_yz_slab_geom(lv, x0, nx, bs.I, bl.d_vgeom, nb, nf * nb, bl.sq);
                 const long long npts = (long long)nx * plane, stride = (long long)bl.slab * plane;
                 if (tc)
