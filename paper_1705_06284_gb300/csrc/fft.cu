@@ -49,6 +49,18 @@ static void allow_smem(K kernel, size_t bytes) {
         FBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
 }
 
+// CTAs of a kernel that fit on the device at once (dynamic shared memory
+// allowed for as needed).
+template <typename K>
+static int resident_ctas(K kernel, int threads, size_t dyn) {
+    int dev = 0, sms = 0, per = 0;
+    FBS_CUDA(cudaGetDevice(&dev));
+    FBS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    FBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    FBS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, dyn));
+    return sms * std::max(1, per);
+}
+
 // ------------------------------------------------------------------ forward
 // z pass: rows r = x*N + y, packed pairs (r0, r0+1) as re/im of one line.
 // Batched evaluations: field blockIdx.y reads fields[blockIdx.y] (when given)
@@ -486,38 +498,81 @@ __global__ void __launch_bounds__(T *LP) inv_z_fast_kernel(const float2 *__restr
 }
 
 // ------------------------------------------------------------------ register z stage
+// cos and sin of 2 pi k / L at compile time: Taylor series on [0, pi/4] after
+// reduction by quarter and eighth turns, so quarter turns are exact.
+constexpr double kPi = 3.14159265358979323846;
+constexpr double ct_series(double x, bool sine) {
+    double term = sine ? x : 1.0, sum = term;
+    for (int n = sine ? 3 : 2; n < 30; n += 2) {
+        term *= -x * x / (n * (n - 1));
+        sum += term;
+    }
+    return sum;
+}
+constexpr double ct_cos(int k, int L) {
+    k %= L;
+    if (k < 0) k += L;
+    if (2 * k > L) k = L - k;                   // cos is even
+    if (4 * k > L) return -ct_cos(L - 2 * k, 2 * L);
+    if (4 * k == L) return 0.0;
+    return 8 * k <= L ? ct_series(2.0 * kPi * k / L, false)
+                      : ct_series(2.0 * kPi * (L - 4 * k) / (4.0 * L), true);
+}
+constexpr double ct_sin(int k, int L) { return ct_cos(4 * k - L, 4 * L); }
+
+// a e^{+2 pi i K / L}
+template <int L, int K>
+__device__ __forceinline__ float2 cmul_unit(float2 a) {
+    if constexpr (K == 0) return a;
+    else if constexpr (4 * K == L) return make_float2(-a.y, a.x);
+    else if constexpr (2 * K == L) return make_float2(-a.x, -a.y);
+    else if constexpr (4 * K == 3 * L) return make_float2(a.y, -a.x);
+    else {
+        constexpr float c = (float)ct_cos(K, L), s = (float)ct_sin(K, L);
+        return make_float2(a.x * c - a.y * s, a.y * c + a.x * s);
+    }
+}
+
 // In-register inverse DFT of length L (e^{+2 pi i nk/L}, unnormalised) of
 // v[0..L), natural order in and out: radix-2/3/4/8 butterflies composed by
 // decimation in time, L = R S with R the largest of 8, 4, 3, 2 dividing L
 // (R < L): S-point sub-transforms of the R interleaved subsequences, the
-// twiddles e^{+2 pi i r k2 / L}, then R-point transforms across them.  The
-// twiddles come from the FP32 table tw of a length NT divisible by L
-// (tw[k] = e^{-2 pi i k/NT}, conjugated).  Every index is a compile-time
-// constant, so the arrays live in registers.
+// twiddles e^{+2 pi i r k2 / L}, then R-point transforms across them.  Every
+// index and twiddle is a compile-time constant: the arrays live in registers
+// and the twiddles are immediates (read from the table, they were half of a
+// thread's load instructions).
 template <int L>
 struct RegRadix {
     static constexpr int R = (L % 8 == 0 && L > 8) ? 8 : (L % 4 == 0 && L > 4) ? 4 : (L % 3 == 0 && L > 3) ? 3 : 2;
 };
 
-template <int L, int NT>
-__device__ __forceinline__ void reg_idft(float2 *v, const float2 *__restrict__ tw) {
+// u[r][k2] *= e^{+2 pi i r k2 / L}, from (r, k2) on in row order.
+template <int L, int R, int r, int k2>
+__device__ __forceinline__ void reg_twiddles(float2 (*u)[L / R]) {
+    if constexpr (r < R) {
+        u[r][k2] = cmul_unit<L, r * k2>(u[r][k2]);
+        if constexpr (k2 + 1 < L / R) reg_twiddles<L, R, r, k2 + 1>(u);
+        else reg_twiddles<L, R, r + 1, 1>(u);
+    }
+}
+
+template <int L>
+__device__ __forceinline__ void reg_idft(float2 *v) {
     if constexpr (L == 1) {
         return;
     } else if constexpr (L == 2 || L == 3 || L == 4 || L == 8) {
         dftR<+1, float, L>(v);
     } else {
         constexpr int R = RegRadix<L>::R, S = L / R;
-        static_assert(R * S == L && NT % L == 0, "length must split over the radices and divide the table");
+        static_assert(R * S == L, "length must split over the radices");
         float2 u[R][S];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
 #pragma unroll
             for (int s = 0; s < S; ++s) u[r][s] = v[r + R * s];
-            reg_idft<S, NT>(u[r], tw);
-#pragma unroll
-            for (int k2 = 1; k2 < S; ++k2)
-                if (r > 0) u[r][k2] = cmulc(u[r][k2], tw[r * k2 * (NT / L)]);  // r k2 < L
+            reg_idft<S>(u[r]);
         }
+        reg_twiddles<L, R, 1, 1>(u);
 #pragma unroll
         for (int k2 = 0; k2 < S; ++k2) {
             float2 w[R];
@@ -530,6 +585,16 @@ __device__ __forceinline__ void reg_idft(float2 *v, const float2 *__restrict__ t
     }
 }
 
+// The twiddles between the two passes, e^{-2 pi i n1 k2/N}, follow the plain
+// table (N entries) as rows [k2][n1]: consecutive threads have consecutive n1
+// and read one line, where the plain table at n1 k2 spreads a warp's 16 values
+// over up to 16 lines (these loads were three quarters of the z stage's L1
+// wavefronts at 512).
+template <int N, int N1>
+__device__ __forceinline__ float2 pass_twiddle(const float2 *__restrict__ tw, int n1, int k2) {
+    return tw[N + k2 * N1 + n1];
+}
+
 // C2R z stage with one shared-memory exchange.  N = N1 N2; a complex line z
 // (two real rows y, y+1 packed as H_y + i H_{y+1}, H the Hermitian completion
 // of the stored half row) is transformed as x[k2 + N2 k1] = sum_{n1}
@@ -539,10 +604,18 @@ __device__ __forceinline__ void reg_idft(float2 *v, const float2 *__restrict__ t
 // in registers (one per k2, N2/T per thread), written straight to the two
 // output rows (consecutive threads hold consecutive k2: coalesced).  T
 // threads per line, LP lines per CTA, T LP a whole number of warps.
+//
+// A CTA runs over row groups (2 LP rows of one plane and bin, contiguous in G):
+// the next group is copied into shared memory (16-byte asynchronous copies)
+// while pass B of this one runs.  Loading the lines straight into registers
+// left the warps waiting for L2 most of the time (long-scoreboard stalls 8.3
+// per issue at 512, 40% of issue slots used).
+// nitems = groups x planes x bins; partial sums of squares [bin][plane][group].
 template <int N, int N1, int N2, int T, int LP>
 __global__ void __launch_bounds__(T *LP) inv_z_reg_kernel(const float2 *__restrict__ G,
-                                                          const BinGeom *__restrict__ geom, int x0,
-                                                          float *__restrict__ out, long long out_bin_stride,
+                                                          const BinGeom *__restrict__ geom, int x0, int nx,
+                                                          int nitems, float *__restrict__ out,
+                                                          long long out_bin_stride,
                                                           double *__restrict__ sumsq_part,
                                                           const float2 *__restrict__ tw) {
     static_assert(N1 * N2 == N && N1 % T == 0 && N2 % T == 0, "threads must divide both passes");
@@ -552,76 +625,103 @@ __global__ void __launch_bounds__(T *LP) inv_z_reg_kernel(const float2 *__restri
     // on consecutive banks
     constexpr int LD = N1 + 1;
     constexpr int LS = N2 * LD + ((T - N2 * LD) % 16 + 16) % 16;
+    constexpr int NG = (N + 2 * LP - 1) / (2 * LP);  // row groups per plane
     __shared__ float2 tile[LP * LS];
     __shared__ float red[(T * LP) / 32];
+    extern __shared__ __align__(16) unsigned char zin_raw[];
+    float2 *const zin = reinterpret_cast<float2 *>(zin_raw);  // 2 LP rows of the group
     const int line = threadIdx.x / T, t = threadIdx.x % T;
-    const int bl = blockIdx.z;
-    const BinGeom g = geom[bl];
-    const int xl = blockIdx.y;
-    const int y = (blockIdx.x * LP + line) * 2;
-    float *ob = out + (long long)bl * out_bin_stride;
-    const bool w0 = y < N, w1 = y + 1 < N;
-    float *o0 = ob + ((long long)xl * N + (w0 ? y : 0)) * N;
-    float *o1 = o0 + N;
-    float acc = 0.f;  // a few squares per thread; FP64 per CTA
-    // an empty bin's rows are never read by any item: nothing to write
-    // (g is the same for the whole CTA, so the barrier inside is uniform)
-    if (!g.empty) {
-        const float2 *in0 = G + g.G_off + ((long long)xl * N + (w0 ? y : 0)) * g.Dzb;
-        const float2 *in1 = in0 + g.Dzb;
-        const int Rz = g.Dzb - 1;  // highest mz held (<= N/2)
-        float2 *Y = tile + line * LS;
+    const auto fetch = [&](int item) {  // the rows of a group, one copy group
+        const int grp = item % NG, r = item / NG, bl = r / nx, xl = r - bl * nx;
+        const int dzb = geom[bl].empty ? 0 : geom[bl].Dzb, y0 = grp * 2 * LP;
+        const float2 *src = G + geom[bl].G_off + ((long long)xl * N + y0) * dzb;
+        const int n16 = min(2 * LP, N - y0) * dzb / 2;  // an even number of rows
+        for (int i = threadIdx.x; i < n16; i += T * LP)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(zin + 2 * i)),
+                         "l"(src + 2 * i)
+                         : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if ((int)blockIdx.x < nitems) fetch(blockIdx.x);
+    for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
+        const int grp = item % NG, rest = item / NG, bl = rest / nx, xl = rest - bl * nx;
+        const int Dzb = geom[bl].Dzb;
+        const int y = (grp * LP + line) * 2;
+        const bool w0 = y < N, w1 = y + 1 < N;
+        float *o0 = out + (long long)bl * out_bin_stride + ((long long)xl * N + (w0 ? y : 0)) * N;
+        float *o1 = o0 + N;
+        float acc = 0.f;  // a few squares per thread; FP64 per CTA
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();  // the group's rows have landed; the tile's readers are done
+        // an empty bin's rows are never read by any item: nothing to write
+        // (the same for the whole CTA, so the barriers inside are uniform)
+        const bool empty = geom[bl].empty;
+        if (!empty) {
+            const float2 *in0 = zin + 2 * line * Dzb;
+            const float2 *in1 = in0 + Dzb;
+            const int Rz = Dzb - 1;  // highest mz held (<= N/2)
+            const int lo = Rz / N1, hi = N2 - (Rz + N1 - 1) / N1;  // n2 in between: no mode, nothing to load
+            float2 *Y = tile + line * LS;
 #pragma unroll 1
-        for (int j = 0; j < N1 / T; ++j) {
-            const int n1 = t + T * j;
-            float2 v[N2];
+            for (int j = 0; j < N1 / T; ++j) {
+                const int n1 = t + T * j;
+                float2 v[N2];
 #pragma unroll
-            for (int n2 = 0; n2 < N2; ++n2) {
-                const int n = n1 + N1 * n2;
-                float2 h1 = make_float2(0.f, 0.f), h2 = make_float2(0.f, 0.f);
-                int m = -1;
-                bool cj = false;
-                if (n <= Rz) m = n;
-                else if (n >= N - Rz) { m = N - n; cj = true; }
-                if (m >= 0) {
-                    if (w0) h1 = in0[m];
-                    if (w1) h2 = in1[m];
-                    if (m == 0 || 2 * m == N) { h1.y = 0.f; h2.y = 0.f; }  // DC and Nyquist of a real row
-                    if (cj) { h1.y = -h1.y; h2.y = -h2.y; }
+                for (int n2 = 0; n2 < N2; ++n2) {
+                    const int n = n1 + N1 * n2;
+                    v[n2] = make_float2(0.f, 0.f);
+                    if (n2 <= lo || n2 >= hi) {  // uniform over the CTA
+                        float2 h1 = make_float2(0.f, 0.f), h2 = make_float2(0.f, 0.f);
+                        int m = -1;
+                        bool cj = false;
+                        if (n <= Rz) m = n;
+                        else if (n >= N - Rz) { m = N - n; cj = true; }
+                        if (m >= 0) {
+                            if (w0) h1 = in0[m];
+                            if (w1) h2 = in1[m];
+                            if (m == 0 || 2 * m == N) { h1.y = 0.f; h2.y = 0.f; }  // DC and Nyquist of a real row
+                            if (cj) { h1.y = -h1.y; h2.y = -h2.y; }
+                        }
+                        v[n2] = make_float2(h1.x - h2.y, h1.y + h2.x);  // H1 + i H2
+                    }
                 }
-                v[n2] = make_float2(h1.x - h2.y, h1.y + h2.x);  // H1 + i H2
-            }
-            reg_idft<N2, N>(v, tw);
+                reg_idft<N2>(v);
 #pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) {
-                float2 val = v[k2];
-                if (k2 > 0) val = cmulc(val, tw[n1 * k2]);  // n1 k2 < N
-                Y[k2 * LD + n1] = val;
+                for (int k2 = 0; k2 < N2; ++k2) {
+                    float2 val = v[k2];
+                    if (k2 > 0) val = cmulc(val, pass_twiddle<N, N1>(tw, n1, k2));
+                    Y[k2 * LD + n1] = val;
+                }
             }
         }
-        __syncthreads();
+        __syncthreads();  // the tile is complete, the input consumed
+        if (item + (int)gridDim.x < nitems) fetch(item + gridDim.x);
+        if (!empty) {
+            const float2 *Y = tile + line * LS;
 #pragma unroll 1
-        for (int j = 0; j < N2 / T; ++j) {
-            const int k2 = t + T * j;
-            float2 v[N1];
+            for (int j = 0; j < N2 / T; ++j) {
+                const int k2 = t + T * j;
+                float2 v[N1];
 #pragma unroll
-            for (int n1 = 0; n1 < N1; ++n1) v[n1] = Y[k2 * LD + n1];
-            reg_idft<N1, N>(v, tw);
+                for (int n1 = 0; n1 < N1; ++n1) v[n1] = Y[k2 * LD + n1];
+                reg_idft<N1>(v);
 #pragma unroll
-            for (int k1 = 0; k1 < N1; ++k1) {
-                const int z = k2 + N2 * k1;
-                if (w0) { o0[z] = v[k1].x; acc = fmaf(v[k1].x, v[k1].x, acc); }
-                if (w1) { o1[z] = v[k1].y; acc = fmaf(v[k1].y, v[k1].y, acc); }
+                for (int k1 = 0; k1 < N1; ++k1) {
+                    const int z = k2 + N2 * k1;
+                    if (w0) { o0[z] = v[k1].x; acc = fmaf(v[k1].x, v[k1].x, acc); }
+                    if (w1) { o1[z] = v[k1].y; acc = fmaf(v[k1].y, v[k1].y, acc); }
+                }
             }
         }
-    }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float s = 0.f;
-        for (int w = 0; w < (T * LP) / 32; ++w) s += red[w];
-        sumsq_part[((long long)bl * N + x0 + xl) * gridDim.x + blockIdx.x] = (double)s;
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            float s = 0.f;
+            for (int w = 0; w < (T * LP) / 32; ++w) s += red[w];
+            sumsq_part[((long long)bl * N + x0 + xl) * NG + grp] = (double)s;
+        }
     }
 }
 
@@ -650,8 +750,8 @@ __global__ void __launch_bounds__(T *LP) inv_y_reg_kernel(const float2 *__restri
     const int xl = blockIdx.y, x = x0 + xl;
     const float2 *in = A + g.A_off + (long long)x * g.Db * g.Dzb;
     const bool full = g.Db == N;  // the bin's box spans the whole axis
-    const int Rb = (g.Db - 1) / 2;
-    const long long mz2 = (long long)mz * mz;
+    const int Rb = full ? N / 2 : (g.Db - 1) / 2;
+    const int mz2 = mz * mz, hi2 = (int)g.thr_hi;          // (at most 3 N^2 / 4)
 #pragma unroll 1
     for (int j = 0; j < N1 / T; ++j) {
         const int n1 = t + T * j;
@@ -659,28 +759,16 @@ __global__ void __launch_bounds__(T *LP) inv_y_reg_kernel(const float2 *__restri
 #pragma unroll
         for (int n2 = 0; n2 < N2; ++n2) {
             const int n = n1 + N1 * n2;
-            int my, jy;
-            if (full) {
-                jy = n;
-                my = n < N / 2 ? n : n - N;
-            } else if (n <= Rb) {
-                jy = n;
-                my = n;
-            } else if (n >= N - Rb) {
-                my = n - N;
-                jy = my + g.Db;
-            } else {
-                jy = -1;
-                my = 0;
-            }
             v[n2] = make_float2(0.f, 0.f);
-            if (col && jy >= 0 && (long long)my * my + mz2 < g.thr_hi) v[n2] = in[(long long)jy * g.Dzb + mz];
+            // (no branch: the loads of all n2 are issued together)
+            const int my = n < N / 2 ? n : n - N;
+            if (col && abs(my) <= Rb && my * my + mz2 < hi2) v[n2] = in[(my < 0 ? my + g.Db : my) * g.Dzb + mz];
         }
-        reg_idft<N2, N>(v, tw);
+        reg_idft<N2>(v);
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) {
             float2 val = v[k2];
-            if (k2 > 0) val = cmulc(val, tw[n1 * k2]);  // n1 k2 < N
+            if (k2 > 0) val = cmulc(val, pass_twiddle<N, N1>(tw, n1, k2));
             tile[(k2 * N1 + n1) * LP + l] = val;
         }
     }
@@ -692,7 +780,7 @@ __global__ void __launch_bounds__(T *LP) inv_y_reg_kernel(const float2 *__restri
         float2 v[N1];
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1) v[n1] = tile[(k2 * N1 + n1) * LP + l];
-        reg_idft<N1, N>(v, tw);
+        reg_idft<N1>(v);
         if (col) {
 #pragma unroll
             for (int k1 = 0; k1 < N1; ++k1) out[(long long)(k2 + N2 * k1) * g.Dzb] = v[k1];
@@ -738,11 +826,11 @@ __global__ void __launch_bounds__(T *LP) fwd_z_reg_kernel(const float *__restric
             const int n = n1 + N1 * n2;
             v[n2] = make_float2(w0 ? f0[n] : 0.f, w1 ? -f1[n] : 0.f);  // conj of the packed line
         }
-        reg_idft<N2, N>(v, tw);
+        reg_idft<N2>(v);
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) {
             float2 val = v[k2];
-            if (k2 > 0) val = cmulc(val, tw[n1 * k2]);  // n1 k2 < N
+            if (k2 > 0) val = cmulc(val, pass_twiddle<N, N1>(tw, n1, k2));
             Y[k2 * LD + n1] = val;
         }
     }
@@ -753,7 +841,7 @@ __global__ void __launch_bounds__(T *LP) fwd_z_reg_kernel(const float *__restric
         const int k2 = t + T * j;
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1) res[j][n1] = Y[k2 * LD + n1];
-        reg_idft<N1, N>(res[j], tw);
+        reg_idft<N1>(res[j]);
     }
     __syncthreads();  // every read of the exchange tile is done
 #pragma unroll
@@ -802,11 +890,11 @@ __global__ void __launch_bounds__(T *LP) inv_x_reg_kernel(const float2 *__restri
     const int l = threadIdx.x % LP, t = threadIdx.x / LP;
     const int mz = jz0 + l;
     const bool col = mz < g.Dzb;
-    const long long r2 = (long long)my * my + (long long)mz * mz;
+    const int r2 = my * my + mz * mz, lo2 = (int)g.thr_lo, hi2 = (int)g.thr_hi;  // at most 3 N^2 / 4 < 2^31
     const float2 *in = box + g.box_off + (long long)box_index(my, bg.D) * bg.Dz + (col ? mz : 0);
     const long long xs = (long long)bg.D * bg.Dz;  // box stride along x
     const bool fullx = bg.D == N;
-    const int R = bg.D / 2;  // the box holds |m_x| <= R when it does not span the axis
+    const int R = fullx ? N / 2 : bg.D / 2;  // the box's largest |m_x|
 #pragma unroll 1
     for (int j = 0; j < N1 / T; ++j) {
         const int n1 = t + T * j;
@@ -814,17 +902,15 @@ __global__ void __launch_bounds__(T *LP) inv_x_reg_kernel(const float2 *__restri
 #pragma unroll
         for (int n2 = 0; n2 < N2; ++n2) {
             const int n = n1 + N1 * n2;
-            const int mx = n < N / 2 ? n : n - N;
-            const int jx = fullx ? n : (mx >= -R && mx <= R ? box_index(mx, bg.D) : -1);
-            const long long s2 = (long long)mx * mx + r2;
             v[n2] = make_float2(0.f, 0.f);
-            if (col && jx >= 0 && s2 >= g.thr_lo && s2 < g.thr_hi) v[n2] = in[(long long)jx * xs];
+            const int mx = n < N / 2 ? n : n - N, s2 = mx * mx + r2;
+            if (col && abs(mx) <= R && s2 >= lo2 && s2 < hi2) v[n2] = in[(long long)(mx < 0 ? mx + bg.D : mx) * xs];
         }
-        reg_idft<N2, N>(v, tw);
+        reg_idft<N2>(v);
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) {
             float2 val = v[k2];
-            if (k2 > 0) val = cmulc(val, tw[n1 * k2]);  // n1 k2 < N
+            if (k2 > 0) val = cmulc(val, pass_twiddle<N, N1>(tw, n1, k2));
             tile[(k2 * N1 + n1) * LP + l] = val;
         }
     }
@@ -837,7 +923,7 @@ __global__ void __launch_bounds__(T *LP) inv_x_reg_kernel(const float2 *__restri
         float2 v[N1];
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1) v[n1] = tile[(k2 * N1 + n1) * LP + l];
-        reg_idft<N1, N>(v, tw);
+        reg_idft<N1>(v);
         if (col) {
 #pragma unroll
             for (int k1 = 0; k1 < N1; ++k1) out[(long long)(k2 + N2 * k1) * os] = v[k1];
@@ -845,7 +931,8 @@ __global__ void __launch_bounds__(T *LP) inv_x_reg_kernel(const float2 *__restri
     }
 }
 
-// Register y-stage configurations: (N, N1, N2, threads per line, columns per CTA).
+// Register y-stage configurations: (N, N1, N2, threads per line, columns per
+// CTA); N1 and N2 are the z stage's, whose twiddle rows they share.
 #define FBS_YREG_LIST(X)        \
     X(64, 8, 8, 8, 8)           \
     X(72, 6, 12, 6, 16)         \
@@ -954,14 +1041,26 @@ static std::vector<double2> twiddles64(int n) {
     return t;
 }
 
+// The FP32 table of a length: n twiddles, then (register stages) the rows
+// [k2][n1] of the twiddles between their two passes.
+static std::vector<float2> twiddles32(const std::vector<double2> &t) {
+    const int n = (int)t.size();
+    std::vector<float2> f(n);
+    for (int k = 0; k < n; ++k) f[k] = make_float2((float)t[k].x, (float)t[k].y);
+#define FBS_TT(len, n1_, n2_, t_, lp_)                                   \
+    if (n == len)                                                        \
+        for (int k2 = 0; k2 < n2_; ++k2)                                 \
+            for (int n1 = 0; n1 < n1_; ++n1) f.push_back(f[n1 * k2]);
+    FBS_ZREG_LIST(FBS_TT)
+#undef FBS_TT
+    return f;
+}
+
 // FP32 twiddles of the input grid (forward transforms).
 void upload_forward_twiddles(Plan &p) {
-    const int N = p.N;
-    const std::vector<double2> tn = twiddles64(N);
-    std::vector<float2> t32(N);
-    for (int k = 0; k < N; ++k) t32[k] = make_float2((float)tn[k].x, (float)tn[k].y);
-    p.d_tw = (float2 *)p.dalloc(N * sizeof(float2));
-    FBS_CUDA(cudaMemcpyAsync(p.d_tw, t32.data(), N * sizeof(float2), cudaMemcpyHostToDevice, p.stream));
+    const std::vector<float2> t32 = twiddles32(twiddles64(p.N));
+    p.d_tw = (float2 *)p.dalloc(t32.size() * sizeof(float2));
+    FBS_CUDA(cudaMemcpyAsync(p.d_tw, t32.data(), t32.size() * sizeof(float2), cudaMemcpyHostToDevice, p.stream));
     FBS_CUDA(cudaStreamSynchronize(p.stream));  // host tables go out of scope
 }
 
@@ -970,11 +1069,10 @@ void upload_forward_twiddles(Plan &p) {
 void upload_eval_twiddles(Plan &p) {
     const int M = p.M;
     const std::vector<double2> tmv = twiddles64(M);
-    std::vector<float2> tm32(M);
-    for (int k = 0; k < M; ++k) tm32[k] = make_float2((float)tmv[k].x, (float)tmv[k].y);
-    p.d_twM = (float2 *)p.dalloc(M * sizeof(float2));
+    const std::vector<float2> tm32 = twiddles32(tmv);
+    p.d_twM = (float2 *)p.dalloc(tm32.size() * sizeof(float2));
     p.d_tw64 = (double2 *)p.dalloc(M * sizeof(double2));
-    FBS_CUDA(cudaMemcpyAsync(p.d_twM, tm32.data(), M * sizeof(float2), cudaMemcpyHostToDevice, p.stream));
+    FBS_CUDA(cudaMemcpyAsync(p.d_twM, tm32.data(), tm32.size() * sizeof(float2), cudaMemcpyHostToDevice, p.stream));
     FBS_CUDA(cudaMemcpyAsync(p.d_tw64, tmv.data(), M * sizeof(double2), cudaMemcpyHostToDevice, p.stream));
     FBS_CUDA(cudaStreamSynchronize(p.stream));  // host tables go out of scope
 }
@@ -1160,12 +1258,16 @@ void launch_inverse_yz_slab_geom(Plan &p, int x0, int nx, float *islab, const Bi
     const int zk = zstage_kind(N);
     if (zk == 2) {
         KTimer t(p, KC_INV_Z);
-        dim3 grid(zstage_row_groups(N), nx, nvb);
+        const int nitems = zstage_row_groups(N) * nx * nvb, dz = max_dzb(p, 0, nb);
         const long long obs = (long long)p.slab * N * N;
-#define FBS_ZR(n, n1, n2, t, lp)                                                   \
-    if (N == n)                                                                    \
-        inv_z_reg_kernel<n, n1, n2, t, lp><<<grid, t * lp, 0, p.stream>>>(          \
-            p.d_G, geom, x0, islab, obs, sq, p.d_twM);
+        // as many CTAs as are resident at once, each over its share of the groups
+#define FBS_ZR(n, n1, n2, t, lp)                                                                            \
+    if (N == n) {                                                                                           \
+        auto k = inv_z_reg_kernel<n, n1, n2, t, lp>;                                                        \
+        const size_t dyn = (size_t)2 * lp * dz * sizeof(float2);                                            \
+        const int G = std::min(nitems, resident_ctas(k, t * lp, dyn));                                      \
+        k<<<G, t * lp, dyn, p.stream>>>(p.d_G, geom, x0, nx, nitems, islab, obs, sq, p.d_twM);              \
+    }
         FBS_ZREG_LIST(FBS_ZR)
 #undef FBS_ZR
         FBS_CUDA(cudaGetLastError());
