@@ -19,6 +19,10 @@ template <> struct V2<double> { typedef double2 t; };
 
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return C{a.x + b.x, a.y + b.y}; }
 template <typename C> __device__ __forceinline__ C csub(C a, C b) { return C{a.x - b.x, a.y - b.y}; }
+// Component by component: after a product, where each add contracts into a
+// fused multiply-add (one rounding, which a packed add would split in two).
+template <typename C> __device__ __forceinline__ C cadd_fma(C a, C b) { return C{a.x + b.x, a.y + b.y}; }
+template <typename C> __device__ __forceinline__ C csub_fma(C a, C b) { return C{a.x - b.x, a.y - b.y}; }
 // FP32: one packed instruction for both components (the same roundings)
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) {
@@ -63,8 +67,8 @@ template <int DIR, typename T, typename C> __device__ __forceinline__ void dft3(
     C t = C{x0.x + c * sum.x, x0.y + c * sum.y};
     C r = mul_i<DIR>(C{s * dif.x, s * dif.y});
     x0 = cadd(x0, sum);
-    x1 = cadd(t, r);
-    x2 = csub(t, r);
+    x1 = cadd_fma(t, r);
+    x2 = csub_fma(t, r);
 }
 
 template <int DIR, typename T, typename C> __device__ __forceinline__ void dft8(C *v) {
@@ -80,12 +84,12 @@ template <int DIR, typename T, typename C> __device__ __forceinline__ void dft8(
     C t3 = C{-h * (o3.x + DIR * o3.y), h * (DIR * o3.x - o3.y)};
     v[0] = cadd(e0, o0);
     v[4] = csub(e0, o0);
-    v[1] = cadd(e1, t1);
-    v[5] = csub(e1, t1);
+    v[1] = cadd_fma(e1, t1);
+    v[5] = csub_fma(e1, t1);
     v[2] = cadd(e2, t2);
     v[6] = csub(e2, t2);
-    v[3] = cadd(e3, t3);
-    v[7] = csub(e3, t3);
+    v[3] = cadd_fma(e3, t3);
+    v[7] = csub_fma(e3, t3);
 }
 
 template <int DIR, typename T, int R, typename C> __device__ __forceinline__ void dftR(C *v) {
