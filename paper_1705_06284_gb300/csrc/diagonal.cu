@@ -22,38 +22,75 @@ namespace fbs {
 
 namespace {
 
-__global__ void field_product_kernel(const float *__restrict__ a, const float *__restrict__ b,
-                                     float *__restrict__ out, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        out[i] = a[i] * b[i];
+// Block (task, quadruplet group): partial sums part[task][q] = w sum_e
+// Re[F_u conj F_v] over the task's half-box modes, F rows u, v of quadruplet q
+// (rows of FA, then of FB).  The modes' values of every row are staged as FP64
+// in shared memory, [mode][row], so each is converted once for all the
+// quadruplets, and a thread spends two FP64 FMAs per mode and quadruplet:
+// what bounds it (two FP64 lanes a cycle per SM: 90 us of FMAs for 123
+// quadruplets at 96^3 and 8 shells).  One block per (shell, quadruplet),
+// converting both rows and multiplying by the weight for every mode, took
+// 1,313 us there, most of it in the blocks of the largest shells; now 155 us.
+constexpr int kDiagThreads = 128;
+
+template <int kDiagQuads>  // quadruplets per thread
+__global__ void __launch_bounds__(kDiagThreads) diag_gram_kernel(
+    const float2 *__restrict__ FA, int na, const float2 *__restrict__ FB, int rows, long long per,
+    const int2 *__restrict__ uv, int nq, const int *__restrict__ idx, const DiagTask *__restrict__ tasks, int chunk,
+    double *__restrict__ part) {
+    extern __shared__ double2 sF[];  // [chunk][rows]
+    const DiagTask t = tasks[blockIdx.x];
+    int2 me[kDiagQuads];
+    double s[kDiagQuads];
+#pragma unroll
+    for (int j = 0; j < kDiagQuads; ++j) {
+        const int q = (blockIdx.y * kDiagQuads + j) * kDiagThreads + threadIdx.x;
+        me[j] = q < nq ? uv[q] : make_int2(0, 0);
+        s[j] = 0.0;
+    }
+    for (int e0 = t.e0; e0 < t.e1; e0 += chunk) {
+        const int n = min(chunk, t.e1 - e0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < rows * n; i += kDiagThreads) {
+            const int r = i / n, k = i - r * n;
+            const float2 v = (r < na ? FA + r * per : FB + (r - na) * per)[idx[e0 + k]];
+            sF[k * rows + r] = make_double2((double)v.x, (double)v.y);
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int k = 0; k < n; ++k) {
+#pragma unroll
+            for (int j = 0; j < kDiagQuads; ++j) {
+                const double2 x = sF[k * rows + me[j].x], y = sF[k * rows + me[j].y];
+                s[j] = fma(x.y, y.y, fma(x.x, y.x, s[j]));
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < kDiagQuads; ++j) {
+        const int q = (blockIdx.y * kDiagQuads + j) * kDiagThreads + threadIdx.x;
+        if (q < nq) part[(long long)blockIdx.x * nq + q] = (double)t.w * s[j];
+    }
 }
 
-// Block (D, q): scale * sum_e w[e] Re[F0[off0 + idx[e]] conj F1[off1 + idx[e]]]
-// over the half-box modes of diagonal shell D (dstart[D]..dstart[D+1]), in
-// FP64 with a fixed-shape tree, into out[qout[q] * nd + D].
-__global__ void __launch_bounds__(256) diag_gram_kernel(const float2 *__restrict__ F0,
-                                                        const float2 *__restrict__ F1,
-                                                        const long long *__restrict__ offs,
-                                                        const int *__restrict__ idx, const float *__restrict__ w,
-                                                        const int *__restrict__ dstart, int nd,
-                                                        const int *__restrict__ qout, double scale,
-                                                        double *__restrict__ out) {
+// out[qout[q] * nd + D] = scale * sum of the shell's task partials: eight
+// threads to a quadruplet, in a fixed order.
+__global__ void __launch_bounds__(256) diag_reduce_kernel(const double *__restrict__ part, int nq,
+                                                          const int *__restrict__ tstart, int nd,
+                                                          const int *__restrict__ qout, double scale,
+                                                          double *__restrict__ out) {
     __shared__ double red[256];
-    const int D = blockIdx.x, q = blockIdx.y;
-    const float2 *x = F0 + offs[2 * q];
-    const float2 *y = F1 + offs[2 * q + 1];
+    const int q = 32 * blockIdx.x + (threadIdx.x & 31), ty = threadIdx.x >> 5, D = blockIdx.y;
     double s = 0.0;
-    for (int e = dstart[D] + threadIdx.x; e < dstart[D + 1]; e += blockDim.x) {
-        const float2 u = x[idx[e]], v = y[idx[e]];
-        s += (double)w[e] * ((double)u.x * (double)v.x + (double)u.y * (double)v.y);
+    if (q < nq) {
+#pragma unroll 4
+        for (int t = tstart[D] + ty; t < tstart[D + 1]; t += 8) s += part[(long long)t * nq + q];
     }
     red[threadIdx.x] = s;
     __syncthreads();
-    for (int k = 128; k > 0; k >>= 1) {
-        if ((int)threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[(long long)qout[q] * nd + D] = scale * red[0];
+    if (ty || q >= nq) return;
+    for (int k = 1; k < 8; ++k) s += red[threadIdx.x + 32 * k];
+    out[(long long)qout[q] * nd + D] = scale * s;
 }
 
 // T_D = cT num_D / N_D (NaN where no closed quadruple has its diagonal in D).
@@ -65,16 +102,27 @@ __global__ void diag_normalise_kernel(const double *__restrict__ num, const doub
 
 }  // namespace
 
-void launch_field_product(Plan &p, const float *a, const float *b, float *out, long long n) {
-    const int blocks = (int)std::min<long long>(4096, (n + 255) / 256);
-    field_product_kernel<<<blocks, 256, 0, p.stream>>>(a, b, out, n);
-    FBS_CUDA(cudaGetLastError());
-}
-
-void launch_diag_gram(Plan &p, const float2 *F0, const float2 *F1, const long long *d_offs, int nq, const int *d_idx,
-                      const float *d_w, const int *d_dstart, int nd, const int *d_qout, double scale, double *out) {
+// Quadruplets uv (rows of FA, then of FB: FB == FA's continuation has nb = 0)
+// over the tasks of every shell; part: ntasks x nq doubles.
+void launch_diag_gram(Plan &p, const float2 *FA, int na, const float2 *FB, int nb, long long per, const int2 *d_uv,
+                      int nq, const int *d_idx, const DiagTask *d_tasks, int ntasks, const int *d_tstart, int nd,
+                      const int *d_qout, double scale, double *part, double *out) {
     if (nq == 0 || nd == 0) return;
-    diag_gram_kernel<<<dim3(nd, nq), 256, 0, p.stream>>>(F0, F1, d_offs, d_idx, d_w, d_dstart, nd, d_qout, scale, out);
+    const int rows = na + nb;
+    // about 64 KB of staged modes (three CTAs per SM), one mode at least
+    const int chunk = std::max(1, std::min(64, (64 * 1024) / (rows * (int)sizeof(double2))));
+    const size_t sm = (size_t)chunk * rows * sizeof(double2);
+    if (sm > 220 * 1024) throw Failure{FBS_ERR_ARG, "too many pair spectra in a group"};
+    if (ntasks > 0) {
+        const int per_block = kDiagThreads * (nq > kDiagThreads ? 2 : 1);
+        const auto kernel = nq > kDiagThreads ? diag_gram_kernel<2> : diag_gram_kernel<1>;
+        FBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        dim3 grid(ntasks, (nq + per_block - 1) / per_block);
+        kernel<<<grid, kDiagThreads, sm, p.stream>>>(FA, na, FB, rows, per, d_uv, nq, d_idx, d_tasks, chunk,
+                                                               part);
+        FBS_CUDA(cudaGetLastError());
+    }
+    diag_reduce_kernel<<<dim3((nq + 31) / 32, nd), 256, 0, p.stream>>>(part, nq, d_tstart, nd, d_qout, scale, out);
     FBS_CUDA(cudaGetLastError());
 }
 

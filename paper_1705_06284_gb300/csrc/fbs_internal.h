@@ -91,6 +91,20 @@ struct FpJob {
     bool built = false;
 };
 
+// Fields that are products of two: field i is base[pairs[i].x] * base[pairs[i].y],
+// `stride` values to a field (launch_forward_grid).
+struct FieldPairs {
+    const float *base;
+    long long stride;
+    const int2 *pairs;
+};
+// Diagonal-resolved trispectrum: modes [e0, e1) of a level's list, all of
+// diagonal shell D and weight w.
+struct DiagTask {
+    int e0, e1, D;
+    float w;
+};
+
 // ---------------------------------------------------------------- timing
 enum KernelClass {
     KC_FWD_Z = 0,
@@ -120,7 +134,7 @@ void launch_forward(Plan &p, const float *d_field, const float *const *d_fields,
                     float2 *ybuf, float2 *box);
 void launch_forward_grid(Plan &p, int N, const BoxGeom &bx, const FftFactors &fN, const float2 *tw,
                          const float *d_field, const float *const *d_fields, int nf, float2 *zbuf, float2 *ybuf,
-                         float2 *box);
+                         float2 *box, const FieldPairs *pairs = nullptr);
 void launch_inverse_x(Plan &p, bool indicator_fp64);
 void launch_inverse_x_geom(Plan &p, const BinGeom *geom, int nb, int nvb);
 void launch_inverse_yz_slab(Plan &p, int x0, int nx, float *islab);
@@ -140,9 +154,9 @@ struct U128 {
 void exact_quad_counts(Plan &p, const double *noct, const std::vector<int> &items, std::vector<U128> &out,
                        const std::vector<long long> *dthr = nullptr, std::vector<U128> *dout = nullptr);
 // diagonal.cu (diagonal-resolved trispectrum)
-void launch_field_product(Plan &p, const float *a, const float *b, float *out, long long n);
-void launch_diag_gram(Plan &p, const float2 *F0, const float2 *F1, const long long *d_offs, int nq, const int *d_idx,
-                      const float *d_w, const int *d_dstart, int nd, const int *d_qout, double scale, double *out);
+void launch_diag_gram(Plan &p, const float2 *FA, int na, const float2 *FB, int nb, long long per, const int2 *d_uv,
+                      int nq, const int *d_idx, const DiagTask *d_tasks, int ntasks, const int *d_tstart, int nd,
+                      const int *d_qout, double scale, double *part, double *out);
 void launch_diag_normalise(Plan &p, const double *num, const double *cnt, long long n, double cT, double *TD);
 // contract.cu (FP64 count sums)
 void launch_count_contraction(Plan &p, const double *noct, int nb_in_group, int bin0,

@@ -65,13 +65,16 @@ static int resident_ctas(K kernel, int threads, size_t dyn) {
 // z pass: rows r = x*N + y, packed pairs (r0, r0+1) as re/im of one line.
 // Batched evaluations: field blockIdx.y reads fields[blockIdx.y] (when given)
 // and writes its own zbuf (stride zstride).
-template <int... Rs>
+// PROD: field blockIdx.y is the product of two (FieldPairs), formed as it is read.
+template <bool PROD, int... Rs>
 __global__ void __launch_bounds__(kThreads) fwd_z_kernel(const float *__restrict__ field_one,
-                                                         const float *const *__restrict__ fields,
+                                                         const float *const *__restrict__ fields, FieldPairs fp,
                                                          float2 *__restrict__ zbuf_all, long long zstride,
                                                          int N, int Dz, int nl, FftFactors f,
                                                          const float2 *__restrict__ tw) {
-    const float *__restrict__ field = fields ? fields[blockIdx.y] : field_one;
+    const float *__restrict__ field = PROD ? fp.base + fp.pairs[blockIdx.y].x * fp.stride
+                                           : fields ? fields[blockIdx.y] : field_one;
+    const float *__restrict__ other = PROD ? fp.base + fp.pairs[blockIdx.y].y * fp.stride : nullptr;
     float2 *__restrict__ zbuf = zbuf_all + (long long)blockIdx.y * zstride;
     extern __shared__ float2 sm[];
     float2 *a = sm;
@@ -84,6 +87,10 @@ __global__ void __launch_bounds__(kThreads) fwd_z_kernel(const float *__restrict
         long long r = row0 + 2 * line;
         float v0 = r < nrows ? field[r * N + z] : 0.f;
         float v1 = r + 1 < nrows ? field[(r + 1) * N + z] : 0.f;
+        if (PROD) {
+            v0 *= r < nrows ? other[r * N + z] : 0.f;
+            v1 *= r + 1 < nrows ? other[(r + 1) * N + z] : 0.f;
+        }
         a[line * ld + z] = make_float2(v0, v1);
     }
     __syncthreads();
@@ -798,9 +805,9 @@ __global__ void __launch_bounds__(T *LP) inv_y_reg_kernel(const float2 *__restri
 // order, and X_r(m) = (Z(m) + conj Z(N-m))/2, X_{r+1}(m) = (Z(m) - conj
 // Z(N-m))/(2i) for the kept m < Dz go to zbuf[r][m].  T threads per line, LP
 // lines per CTA; batched evaluations read fields[blockIdx.y].
-template <int N, int N1, int N2, int T, int LP>
+template <int N, int N1, int N2, int T, int LP, bool PROD>
 __global__ void __launch_bounds__(T *LP) fwd_z_reg_kernel(const float *__restrict__ field_one,
-                                                          const float *const *__restrict__ fields,
+                                                          const float *const *__restrict__ fields, FieldPairs fp,
                                                           float2 *__restrict__ zbuf_all, long long zstride, int Dz,
                                                           const float2 *__restrict__ tw) {
     static_assert(N1 * N2 == N && N1 % T == 0 && N2 % T == 0, "threads must divide both passes");
@@ -808,7 +815,9 @@ __global__ void __launch_bounds__(T *LP) fwd_z_reg_kernel(const float *__restric
     constexpr int LD = N1 + 1;
     constexpr int LS = N2 * LD + ((T - N2 * LD) % 16 + 16) % 16;  // >= N: the tile also holds the line
     __shared__ float2 tile[LP * LS];
-    const float *__restrict__ field = fields ? fields[blockIdx.y] : field_one;
+    const float *__restrict__ field = PROD ? fp.base + fp.pairs[blockIdx.y].x * fp.stride
+                                           : fields ? fields[blockIdx.y] : field_one;
+    const long long oth = PROD ? (fp.pairs[blockIdx.y].y - fp.pairs[blockIdx.y].x) * fp.stride : 0;
     float2 *__restrict__ zbuf = zbuf_all + (long long)blockIdx.y * zstride;
     const int line = threadIdx.x / T, t = threadIdx.x % T;
     const long long nrows = (long long)N * N;
@@ -824,7 +833,12 @@ __global__ void __launch_bounds__(T *LP) fwd_z_reg_kernel(const float *__restric
 #pragma unroll
         for (int n2 = 0; n2 < N2; ++n2) {
             const int n = n1 + N1 * n2;
-            v[n2] = make_float2(w0 ? f0[n] : 0.f, w1 ? -f1[n] : 0.f);  // conj of the packed line
+            float a = w0 ? f0[n] : 0.f, b = w1 ? -f1[n] : 0.f;  // conj of the packed line
+            if (PROD) {
+                a *= w0 ? f0[n + oth] : 0.f;
+                b *= w1 ? f1[n + oth] : 0.f;
+            }
+            v[n2] = make_float2(a, b);
         }
         reg_idft<N2>(v);
 #pragma unroll
@@ -1111,17 +1125,18 @@ void launch_forward(Plan &p, const float *d_field, const float *const *d_fields,
 // evaluation grid for products of shell fields), pruned to the box bx.
 void launch_forward_grid(Plan &p, int N, const BoxGeom &bx, const FftFactors &fN, const float2 *tw,
                          const float *d_field, const float *const *d_fields, int nf, float2 *zbuf, float2 *ybuf,
-                         float2 *box) {
+                         float2 *box, const FieldPairs *pairs) {
+    const FieldPairs fp = pairs ? *pairs : FieldPairs{nullptr, 0, nullptr};
     const int D = bx.D, Dz = bx.Dz;
     const long long zs = (long long)N * N * Dz, ys = (long long)N * D * Dz, bs = (long long)D * D * Dz;
     const int nl = lines_per_cta<float>(N);
     const size_t sm = 2 * (size_t)nl * (N + 1) * sizeof(float2);
-    auto kz = fwd_z_kernel<>;
+    auto kz = pairs ? fwd_z_kernel<true> : fwd_z_kernel<false>;
     auto ky = fwd_y_kernel<>;
     auto kx = fwd_x_kernel<>;
 #define FBS_PICK(n, ...)                 \
     if (N == n) {                        \
-        kz = fwd_z_kernel<__VA_ARGS__>;  \
+        kz = pairs ? fwd_z_kernel<true, __VA_ARGS__> : fwd_z_kernel<false, __VA_ARGS__>; \
         ky = fwd_y_kernel<__VA_ARGS__>;  \
         kx = fwd_x_kernel<__VA_ARGS__>;  \
     }
@@ -1136,15 +1151,19 @@ void launch_forward_grid(Plan &p, int N, const BoxGeom &bx, const FftFactors &fN
         const int lp = zreg_lines(N);
         if (lp > 0 && !(fenv && !strcmp(fenv, "smem"))) {
             dim3 grid((int)((rows + 2 * lp - 1) / (2 * lp)), nf);
-#define FBS_FZ(n, n1, n2, t_, lp_)                                                    \
-    if (N == n) fwd_z_reg_kernel<n, n1, n2, t_, lp_><<<grid, t_ * lp_, 0, p.stream>>>( \
-                    d_field, d_fields, zbuf, zs, Dz, tw);
+#define FBS_FZ(n, n1, n2, t_, lp_)                                                                              \
+    if (N == n && pairs)                                                                                        \
+        fwd_z_reg_kernel<n, n1, n2, t_, lp_, true><<<grid, t_ * lp_, 0, p.stream>>>(nullptr, nullptr, fp, zbuf, \
+                                                                                    zs, Dz, tw);                \
+    else if (N == n)                                                                                            \
+        fwd_z_reg_kernel<n, n1, n2, t_, lp_, false><<<grid, t_ * lp_, 0, p.stream>>>(d_field, d_fields, fp,     \
+                                                                                     zbuf, zs, Dz, tw);
             FBS_ZREG_LIST(FBS_FZ)
 #undef FBS_FZ
         } else {
             allow_smem(kz, sm);
             dim3 grid((int)((rows + 2 * nl - 1) / (2 * nl)), nf);
-            kz<<<grid, kThreads, sm, p.stream>>>(d_field, d_fields, zbuf, zs, N, Dz, nl, fN, tw);
+            kz<<<grid, kThreads, sm, p.stream>>>(d_field, d_fields, fp, zbuf, zs, N, Dz, nl, fN, tw);
         }
         FBS_CUDA(cudaGetLastError());
     }

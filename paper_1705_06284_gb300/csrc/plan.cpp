@@ -1163,8 +1163,11 @@ static void run_batch(Plan &p, const float *const *fields, int nf) {
 // quadruplets (split (a, b) | (c, d)).
 struct DiagLevel {
     BoxGeom bx{};
-    int *d_idx = nullptr, *d_dstart = nullptr;
-    float *d_w = nullptr;
+    int *d_idx = nullptr, *d_tstart = nullptr;  // modes by shell and weight; first task of every shell
+    DiagTask *d_tasks = nullptr;
+    int ntasks = 0;
+    int2 *d_pairs = nullptr, *d_uv = nullptr;   // bins of every pair; pair rows of every quadruplet
+    int *d_qout = nullptr;
     BinGeom *d_geom_full = nullptr;
     long long G_full = 0;
     std::vector<std::pair<int, int>> pairs;
@@ -1223,8 +1226,7 @@ static void set_diagonal(Plan &p, const double *edges, int nd) {
         dl.bx.R = Rq;
         dl.bx.D = 2 * Rq + 1 > M ? M : 2 * Rq + 1;
         dl.bx.Dz = std::min(Rq, M / 2) + 1;
-        std::vector<std::vector<int>> li(nd);
-        std::vector<std::vector<float>> lw(nd);
+        std::vector<std::vector<int>> li(2 * nd);  // modes of (shell, weight 2), (shell, weight 1)
         for (int jx = 0; jx < dl.bx.D; ++jx)
             for (int jy = 0; jy < dl.bx.D; ++jy)
                 for (int jz = 0; jz < dl.bx.Dz; ++jz) {
@@ -1232,19 +1234,29 @@ static void set_diagonal(Plan &p, const double *edges, int nd) {
                     const long long s2 = qx * qx + qy * qy + (long long)jz * jz;
                     if (s2 < thr[0] || s2 >= top) continue;
                     const int D = (int)(std::upper_bound(thr.begin(), thr.end(), s2) - thr.begin()) - 1;
-                    li[D].push_back((int)(((long long)jx * dl.bx.D + jy) * dl.bx.Dz + jz));
-                    lw[D].push_back(jz == 0 || 2 * jz == M ? 1.f : 2.f);
+                    li[2 * D + (jz == 0 || 2 * jz == M)].push_back(
+                        (int)(((long long)jx * dl.bx.D + jy) * dl.bx.Dz + jz));
                 }
+        // tasks of one shell and weight, 256 modes or what makes about 1,200 of them
+        size_t total = 0;
+        for (const auto &v : li) total += v.size();
+        const size_t step = std::max<size_t>(256, (total + 1199) / 1200);
         std::vector<int> idx, start(1, 0);
-        std::vector<float> w;
+        std::vector<DiagTask> tasks;
         for (int D = 0; D < nd; ++D) {
-            idx.insert(idx.end(), li[D].begin(), li[D].end());
-            w.insert(w.end(), lw[D].begin(), lw[D].end());
-            start.push_back((int)idx.size());
+            for (int k = 0; k < 2; ++k) {
+                const auto &v = li[2 * D + k];
+                for (size_t e = 0; e < v.size(); e += step)
+                    tasks.push_back(DiagTask{(int)(idx.size() + e), (int)(idx.size() + std::min(v.size(), e + step)), D,
+                                             k ? 1.f : 2.f});
+                idx.insert(idx.end(), v.begin(), v.end());
+            }
+            start.push_back((int)tasks.size());
         }
         dl.d_idx = upload(lv, idx);
-        dl.d_w = upload(lv, w);
-        dl.d_dstart = upload(lv, start);
+        dl.d_tasks = upload(lv, tasks);
+        dl.ntasks = (int)tasks.size();
+        dl.d_tstart = upload(lv, start);
         std::vector<BinGeom> g = lv.geom;
         long long goff = 0;
         for (int b = 0; b < lv.nbins; ++b) {
@@ -1265,6 +1277,12 @@ static void set_diagonal(Plan &p, const double *edges, int nd) {
                 }
                 dl.qp[i][h] = it->second;
             }
+        std::vector<int2> pv, uv;
+        for (const auto &k : dl.pairs) pv.push_back(make_int2(k.first, k.second));
+        for (const auto &k : dl.qp) uv.push_back(make_int2(k[0], k[1]));
+        dl.d_pairs = upload(lv, pv);
+        dl.d_uv = upload(lv, uv);
+        dl.d_qout = upload(lv, lv.gquad);
         FBS_CUDA(cudaStreamSynchronize(lv.stream));  // the host tables go out of scope
     }
     ds->cnt.resize(ds->cnt128.size());
@@ -1276,7 +1294,8 @@ static void set_diagonal(Plan &p, const double *edges, int nd) {
 }
 
 // Shell fields of every bin of a level on its whole grid, then per group of
-// pairs the forward transforms of their products, then the Gram products.
+// pairs the forward transforms of their products (many to a launch, the
+// product formed as the z pass reads it), then the Gram products.
 static void run_diagonal(Plan &p, const float *field) {
     DiagState &ds = *reinterpret_cast<DiagState *>(p.diag);
     const int nd = ds.nd;
@@ -1307,63 +1326,68 @@ static void run_diagonal(Plan &p, const float *field) {
         lv.d_G = G0;
         lv.slab = slab0;
         const long long per = (long long)dl.bx.D * dl.bx.D * dl.bx.Dz;  // complex elements of one pair spectrum
-        const int K = (int)std::max<long long>(1, std::min<long long>(np, (4LL << 30) / (per * 8)));
+        // pair spectra in groups of 4 GiB at most, few enough to stage one mode of two groups
+        const int K = (int)std::max<long long>(1, std::min<long long>({np, 6000, (4LL << 30) / (per * 8)}));
         const int ng = (np + K - 1) / K;
-        AsyncBuf prod((size_t)M3 * sizeof(float), p.stream, "diagonal scratch");
-        AsyncBuf zb((size_t)M * M * dl.bx.Dz * sizeof(float2), p.stream, "diagonal scratch");
-        AsyncBuf yb((size_t)M * dl.bx.D * dl.bx.Dz * sizeof(float2), p.stream, "diagonal scratch");
+        // forward transforms of as many products at once as a gigabyte of scratch holds
+        const long long fwd = (long long)M * M * dl.bx.Dz + (long long)M * dl.bx.D * dl.bx.Dz;
+        int F = (int)std::max<long long>(1, std::min<long long>(std::min(np, K), (1LL << 30) / (fwd * 8)));
+        const auto scratch = [&] {
+            return std::unique_ptr<AsyncBuf>(new AsyncBuf((size_t)F * fwd * sizeof(float2), p.stream, "diagonal scratch"));
+        };
+        std::unique_ptr<AsyncBuf> zy;
+        try {
+            zy = scratch();
+        } catch (const Failure &) {  // (no room for that: one at a time)
+            F = 1;
+            zy = scratch();
+        }
+        float2 *const zb = zy->as<float2>(), *const yb = zb + (long long)F * M * M * dl.bx.Dz;
         AsyncBuf FA((size_t)std::min(np, K) * per * sizeof(float2), p.stream, "pair spectra");
         AsyncBuf FB(ng > 1 ? (size_t)K * per * sizeof(float2) : 16, p.stream, "pair spectra");
-        const float *If = Ifull.as<float>();
+        const int nql = (int)lv.nquad.size();
+        AsyncBuf part((size_t)std::max(1, dl.ntasks) * nql * sizeof(double), p.stream, "diagonal scratch");
         auto compute = [&](int g, float2 *dst) {
-            for (int j = g * K; j < std::min(np, (g + 1) * K); ++j) {
-                launch_field_product(lv, If + (long long)dl.pairs[j].first * M3, If + (long long)dl.pairs[j].second * M3,
-                                     prod.as<float>(), M3);
-                launch_forward_grid(lv, M, dl.bx, lv.fM, lv.d_twM, prod.as<float>(), nullptr, 1, zb.as<float2>(),
-                                    yb.as<float2>(), dst + (long long)(j - g * K) * per);
+            const int end = std::min(np, (g + 1) * K);
+            for (int j = g * K; j < end; j += F) {
+                const FieldPairs fp{Ifull.as<float>(), M3, dl.d_pairs + j};
+                launch_forward_grid(lv, M, dl.bx, lv.fM, lv.d_twM, nullptr, nullptr, std::min(F, end - j), zb, yb,
+                                    dst + (long long)(j - g * K) * per, &fp);
             }
         };
         const double scale = 1.0 / ((double)M3 * (double)M3);  // DFT_M of a pair product is M^3 F_ab
-        const int nql = (int)lv.nquad.size();
+        if (ng == 1) {
+            compute(0, FA.as<float2>());
+            launch_diag_gram(lv, FA.as<float2>(), np, nullptr, 0, per, dl.d_uv, nql, dl.d_idx, dl.d_tasks, dl.ntasks,
+                             dl.d_tstart, nd, dl.d_qout, scale, part.as<double>(), ds.d_num);
+            continue;
+        }
         for (int gi = 0; gi < ng; ++gi) {
             compute(gi, FA.as<float2>());
+            const int na = std::min(np, (gi + 1) * K) - gi * K;
             for (int gj = gi; gj < ng; ++gj) {
-                std::vector<long long> offs;
+                const int nbr = gj == gi ? 0 : std::min(np, (gj + 1) * K) - gj * K;
+                std::vector<int2> uv;
                 std::vector<int> qout;
                 for (int i = 0; i < nql; ++i) {
-                    const int g0 = dl.qp[i][0] / K, g1 = dl.qp[i][1] / K;
-                    int u, v;
-                    if (g0 == gi && g1 == gj) {
-                        u = dl.qp[i][0];
-                        v = dl.qp[i][1];
-                    } else if (g1 == gi && g0 == gj) {
-                        u = dl.qp[i][1];
-                        v = dl.qp[i][0];
-                    } else {
-                        continue;
-                    }
-                    offs.push_back((long long)(u - gi * K) * per);
-                    offs.push_back((long long)(v - gj * K) * per);
+                    int u = dl.qp[i][0], v = dl.qp[i][1];
+                    if (u / K > v / K) std::swap(u, v);
+                    if (u / K != gi || v / K != gj) continue;
+                    uv.push_back(make_int2(u - gi * K, v - gj * K + (gj == gi ? 0 : na)));
                     qout.push_back(lv.gquad[i]);
                 }
                 if (qout.empty()) continue;
-                const float2 *Bp = FA.as<float2>();
-                if (gj != gi) {
-                    compute(gj, FB.as<float2>());
-                    Bp = FB.as<float2>();
-                }
-                for (size_t c0 = 0; c0 < qout.size(); c0 += 65535) {
-                    const int nc = (int)std::min<size_t>(65535, qout.size() - c0);
-                    AsyncBuf d_offs((size_t)nc * 2 * sizeof(long long), p.stream, "diagonal scratch");
-                    AsyncBuf d_q((size_t)nc * sizeof(int), p.stream, "diagonal scratch");
-                    FBS_CUDA(cudaMemcpyAsync(d_offs.ptr, offs.data() + 2 * c0, (size_t)nc * 2 * sizeof(long long),
-                                             cudaMemcpyHostToDevice, p.stream));
-                    FBS_CUDA(cudaMemcpyAsync(d_q.ptr, qout.data() + c0, (size_t)nc * sizeof(int),
-                                             cudaMemcpyHostToDevice, p.stream));
-                    launch_diag_gram(lv, FA.as<float2>(), Bp, d_offs.as<long long>(), nc, dl.d_idx, dl.d_w,
-                                     dl.d_dstart, nd, d_q.as<int>(), scale, ds.d_num);
-                    FBS_CUDA(cudaStreamSynchronize(p.stream));  // offs and qout go out of scope
-                }
+                if (gj != gi) compute(gj, FB.as<float2>());
+                AsyncBuf d_uv(uv.size() * sizeof(int2), p.stream, "diagonal scratch");
+                AsyncBuf d_q(qout.size() * sizeof(int), p.stream, "diagonal scratch");
+                FBS_CUDA(cudaMemcpyAsync(d_uv.ptr, uv.data(), uv.size() * sizeof(int2), cudaMemcpyHostToDevice,
+                                         p.stream));
+                FBS_CUDA(cudaMemcpyAsync(d_q.ptr, qout.data(), qout.size() * sizeof(int), cudaMemcpyHostToDevice,
+                                         p.stream));
+                launch_diag_gram(lv, FA.as<float2>(), na, FB.as<float2>(), nbr, per, d_uv.as<int2>(), (int)uv.size(),
+                                 dl.d_idx, dl.d_tasks, dl.ntasks, dl.d_tstart, nd, d_q.as<int>(), scale,
+                                 part.as<double>(), ds.d_num);
+                FBS_CUDA(cudaStreamSynchronize(p.stream));  // uv and qout go out of scope
             }
         }
     }
