@@ -954,11 +954,14 @@ __global__ void __launch_bounds__(T *LP) inv_x_reg_kernel(const float2 *__restri
     X(108, 9, 12, 3, 32)        \
     X(128, 8, 16, 8, 8)         \
     X(144, 12, 12, 12, 8)       \
+    X(162, 9, 18, 9, 32)        \
     X(192, 8, 24, 8, 8)         \
     X(216, 12, 18, 6, 16)       \
     X(256, 16, 16, 16, 8)       \
     X(288, 12, 24, 12, 8)       \
+    X(324, 18, 18, 18, 16)      \
     X(384, 16, 24, 8, 8)        \
+    X(432, 12, 36, 12, 8)       \
     X(512, 16, 32, 16, 8)
 
 // Register z-stage configurations: (N, N1, N2, threads per line, lines per
@@ -971,11 +974,14 @@ __global__ void __launch_bounds__(T *LP) inv_x_reg_kernel(const float2 *__restri
     X(108, 9, 12, 3, 32)        \
     X(128, 8, 16, 8, 16)        \
     X(144, 12, 12, 12, 8)       \
+    X(162, 9, 18, 9, 32)        \
     X(192, 8, 24, 8, 16)        \
     X(216, 12, 18, 6, 16)       \
     X(256, 16, 16, 16, 8)       \
     X(288, 12, 24, 12, 8)       \
+    X(324, 18, 18, 18, 16)      \
     X(384, 16, 24, 8, 8)        \
+    X(432, 12, 36, 12, 8)       \
     X(512, 16, 32, 16, 8)
 
 // Fast z-stage configurations: (N, threads per line, lines per CTA, radices).
