@@ -278,12 +278,17 @@ __global__ void normalise_kernel(const double *__restrict__ tnum, const int64_t 
 
 // ------------------------------------------------------------------ connected trispectrum
 // Per-shell moments of the spectrum box (the forward output): for bin b
-// (blockIdx.y) and one of gridDim.x chunks of its sub-box |m_j| <= R_b,
+// (blockIdx.y), over the rows (m_x, m_y) of its sub-box |m_j| <= R_b that
+// this one of gridDim.x chunks takes,
 //   S2 = sum |D|^2, S4 = sum |D|^4 over the shell's modes,
 //   Z4 = sum D^4 over its self-conjugate modes (m = -m mod N, D real there).
 // The box holds mz >= 0 only: a mode with 0 < mz < N/2 stands for itself and
 // its conjugate at -mz (weight 2); the planes mz = 0 and mz = N/2 hold both.
 // One partial per (bin, chunk, moment), from a fixed-shape block reduction.
+// A warp takes a row, rows are dealt out round robin (the widest shell holds
+// most of the modes) and rows outside the shell cost one test.  Measured at
+// 162, 9 logarithmic bins: 65 -> 22 us against 16 chunks of modes, each
+// found by 64-bit divisions.
 __global__ void __launch_bounds__(256) shell_moments_kernel(const float2 *__restrict__ box, BoxGeom bg,
                                                             const BinGeom *__restrict__ gb,
                                                             double *__restrict__ part) {
@@ -292,22 +297,40 @@ __global__ void __launch_bounds__(256) shell_moments_kernel(const float2 *__rest
     const BinGeom g = gb[b];
     double s2 = 0.0, s4 = 0.0, z4 = 0.0;
     if (!g.empty) {
-        const long long n = (long long)g.Db * g.Db * g.Dzb;
-        const long long c0 = n * blockIdx.x / gridDim.x, c1 = n * (blockIdx.x + 1) / gridDim.x;
-        for (long long e = c0 + threadIdx.x; e < c1; e += blockDim.x) {
-            const int jz = (int)(e % g.Dzb);
-            const long long r = e / g.Dzb;
-            const int jy = (int)(r % g.Db), jx = (int)(r / g.Db);
-            const int mx = box_freq(jx, g.Db, N), my = box_freq(jy, g.Db, N), mz = jz;
-            const long long s = (long long)mx * mx + (long long)my * my + (long long)mz * mz;
-            if (s < g.thr_lo || s >= g.thr_hi) continue;
-            const float2 d = box[((long long)box_index(mx, bg.D) * bg.D + box_index(my, bg.D)) * bg.Dz + mz];
-            const double a2 = (double)d.x * d.x + (double)d.y * d.y;
-            const double w = (mz == 0 || 2 * mz == N) ? 1.0 : 2.0;
-            s2 += w * a2;
-            s4 += w * a2 * a2;
-            const bool scx = mx == 0 || 2 * mx == -N, scy = my == 0 || 2 * my == -N;
-            if (scx && scy && (mz == 0 || 2 * mz == N)) z4 += (double)d.x * d.x * d.x * d.x;
+        const int lane = threadIdx.x & 31, rows = g.Db * g.Db, step = gridDim.x * 8;
+        for (int r0 = blockIdx.x * 8 + (threadIdx.x >> 5); r0 < rows; r0 += 4 * step) {
+            const float2 *row[4];  // four rows in flight
+            int r2[4];             // at most N^2 / 2; -1: no row
+            bool sc[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int r = r0 + q * step, jx = r / g.Db, jy = r - jx * g.Db;
+                const int mx = box_freq(jx, g.Db, N), my = box_freq(jy, g.Db, N);
+                r2[q] = r < rows ? mx * mx + my * my : -1;
+                row[q] = box + ((long long)box_index(mx, bg.D) * bg.D + box_index(my, bg.D)) * bg.Dz;
+                sc[q] = (mx == 0 || 2 * mx == -N) && (my == 0 || 2 * my == -N);
+            }
+            for (int mz = lane; mz < g.Dzb; mz += 32) {
+                const bool plane = mz == 0 || 2 * mz == N;
+                const double w = plane ? 1.0 : 2.0;
+                float2 d[4];
+                bool on[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const long long s = (long long)r2[q] + mz * mz;
+                    d[q] = make_float2(0.f, 0.f);
+                    on[q] = r2[q] >= 0 && s >= g.thr_lo && s < g.thr_hi;
+                    if (on[q]) d[q] = row[q][mz];
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (!on[q]) continue;
+                    const double a2 = (double)d[q].x * d[q].x + (double)d[q].y * d[q].y;
+                    s2 += w * a2;
+                    s4 += w * a2 * a2;
+                    if (sc[q] && plane) z4 += (double)d[q].x * d[q].x * d[q].x * d[q].x;
+                }
+            }
         }
     }
     red[0][threadIdx.x] = s2;
@@ -330,28 +353,34 @@ __global__ void __launch_bounds__(256) shell_moments_kernel(const float2 *__rest
 //   otherwise     : 0,
 // Tc = V^3/N_pix^4 (qnum/N_pix - paired sum) / N_conn, N_conn the unpaired
 // count (plan time).  NaN where a wait timed out or no unpaired quadruple is left.
-__global__ void connected_kernel(const double *__restrict__ qnum, const int *__restrict__ quad,
-                                 const double *__restrict__ nconn, int nquad,
-                                 const double *__restrict__ mom_part, int chunks, double L, int N,
-                                 double *__restrict__ Tc, const int *__restrict__ err) {
+//
+// Every block first adds up the chunks of all moments, a warp per sum in a
+// fixed order, into shared memory (one thread per quadruplet adding them from
+// global memory was a chain of up to 3 x 16 dependent loads and adds).
+__global__ void __launch_bounds__(256) connected_kernel(const double *__restrict__ qnum, const int *__restrict__ quad,
+                                                        const double *__restrict__ nconn, int nquad,
+                                                        const double *__restrict__ mom_part, int nbins, double L,
+                                                        int N, double *__restrict__ Tc, const int *__restrict__ err) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    double *const mom = reinterpret_cast<double *>(smraw);  // [bin][moment]
+    for (int m = threadIdx.x >> 5; m < 3 * nbins; m += 8) {
+        const double *src = mom_part + (long long)(m / 3) * kMomChunks * 3 + m % 3;
+        double s = 0.0;
+#pragma unroll
+        for (int j = 0; j < kMomChunks / 32; ++j) s += src[3 * ((threadIdx.x & 31) + 32 * j)];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 31) == 0) mom[m] = s;
+    }
+    __syncthreads();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nquad) return;
     const double V = L * L * L, npix = (double)N * N * N;
     const double cT = V * V * V / (npix * npix * npix * npix);
     const int a = quad[4 * i], b = quad[4 * i + 1], c = quad[4 * i + 2], d = quad[4 * i + 3];
-    auto mom = [&](int bin, int k) {  // chunks summed in a fixed order
-        double s = 0.0;
-        for (int j = 0; j < chunks; ++j) s += mom_part[((long long)bin * chunks + j) * 3 + k];
-        return s;
-    };
     double paired = 0.0;
     if (a == b && c == d) {
-        if (a != c) {
-            paired = mom(a, 0) * mom(c, 0);
-        } else {
-            const double s2 = mom(a, 0);
-            paired = 3.0 * s2 * s2 - 3.0 * mom(a, 1) + mom(a, 2);
-        }
+        const double s2 = mom[3 * a];
+        paired = a != c ? s2 * mom[3 * c] : 3.0 * s2 * s2 - 3.0 * mom[3 * a + 1] + mom[3 * a + 2];
     }
     const bool bad = (err && *err) || !(nconn[i] > 0.0);
     Tc[i] = bad ? nan("") : cT * (qnum[i] / npix - paired) / nconn[i];
@@ -359,14 +388,14 @@ __global__ void connected_kernel(const double *__restrict__ qnum, const int *__r
 
 void launch_connected(Plan &p, double *d_Tc) {
     KTimer tm(p, KC_REDUCE);
-    const int chunks = 16;
-    dim3 grid(chunks, p.nbins);
+    dim3 grid(kMomChunks, p.nbins);
     shell_moments_kernel<<<grid, 256, 0, p.stream>>>(p.d_box, p.box, p.d_geom, p.d_mom_part);
     FBS_CUDA(cudaGetLastError());
     const int nq = (int)p.nquad.size();
     if (nq == 0) return;
-    connected_kernel<<<(nq + 255) / 256, 256, 0, p.stream>>>(
-        p.d_qnum, p.d_quadtab, p.d_nconn, nq, p.d_mom_part, chunks, p.L, p.N, d_Tc,
+    const size_t sm = (size_t)p.nbins * 3 * sizeof(double);  // at most 128 bins
+    connected_kernel<<<(nq + 255) / 256, 256, sm, p.stream>>>(
+        p.d_qnum, p.d_quadtab, p.d_nconn, nq, p.d_mom_part, p.nbins, p.L, p.N, d_Tc,
         p.precision != FBS_PREC_FP32 ? tc_error_flag(p) : nullptr);
     FBS_CUDA(cudaGetLastError());
 }

@@ -187,6 +187,7 @@ void launch_normalise(Plan &root, bool quads);
 void launch_normalise_batch(Plan &root, bool quads, int nf, const double *tnum, const double *sumsq, double *B,
                             double *P);
 // Connected trispectrum of the last evaluation into d_Tc[nquad] (root).
+constexpr int kMomChunks = 64;  // partials per bin of the shell moments
 void launch_connected(Plan &root, double *d_Tc);
 std::vector<int> fast_grids();  // grids with compile-time-radix kernels for every inverse stage
 void prepare_fp32(Plan &level, bool trip, bool quads);

@@ -922,7 +922,7 @@ static void create_plan(Plan &p, const double *edges, const void *blob = nullptr
         p.d_quadtab = upload(p, p.quad);
         p.d_Tc = (double *)p.dalloc((size_t)nquad * sizeof(double));
     }
-    p.d_mom_part = (double *)p.dalloc((size_t)nb * 16 * 3 * sizeof(double));
+    p.d_mom_part = (double *)p.dalloc((size_t)nb * kMomChunks * 3 * sizeof(double));
     FBS_CUDA(cudaStreamSynchronize(p.stream));
 }
 
