@@ -62,7 +62,9 @@ typedef enum {
  * in every mode; counts are FP64 in every mode. */
 enum {
     FBS_PREC_FP32 = 0,    /* CUDA-core FP32 products, FP64 cross-block sums      */
-    FBS_PREC_BF16X3 = 1,  /* tcgen05 tensor cores, BF16 hi/lo split, 3 products  */
+    FBS_PREC_BF16X3 = 1,  /* tcgen05 tensor cores, BF16 hi/lo split: hi*hi, hi*lo
+                           * and lo*hi (lo*lo too in triplet jobs of the shared-
+                           * operand contraction and of FBS_OPT_TC_STACK)       */
     FBS_PREC_BF16 = 2     /* tcgen05 tensor cores, plain BF16 (error reported)   */
 };
 
@@ -169,7 +171,14 @@ fbs_status fbs_plan_shells(const fbs_plan *plan, int64_t *sizes, int64_t *thr);
 /* Change the contraction precision of an existing plan (FBS_PREC_*). */
 fbs_status fbs_plan_set_precision(fbs_plan *plan, int precision);
 
-/* Plan options (fbs_plan_set_option). */
+/* Plan options (fbs_plan_set_option).  With every FBS_OPT_TC_* option but
+ * FBS_OPT_TC_WAIT_LIMIT at its default, BF16x3 triplet sums and fused
+ * triplet + quadruplet sums run on the shared-operand contraction (both
+ * operands' rows formed once in shared memory) where the job's rows fit it.
+ * Any of FBS_OPT_TC_WIDE, _ROLES, _CHUNK, _PAIRS, _MERGE, _BSTAGES, _BFROMA and
+ * _STACK set, a job that does not fit, plain BF16 and the connected
+ * trispectrum run on the tensor-memory contraction that these options describe.
+ * The two agree within the precision's rounding. */
 enum {
     FBS_OPT_TC_WIDE = 1, /* 0: tensor-core contraction with the pair products as
                            operand A (M = 128 outer pairs, N = bins; default);
@@ -322,6 +331,8 @@ fbs_status fbs_trispectrum_connected(fbs_plan *plan, const float *field, double 
  * pipeline step of that launch, its operand-A stages in tensor memory, its
  * operand-B stages and its field stages in shared memory, the number of
  * inner pair rows it took from operand A (FBS_OPT_TC_BFROMA; 0: none)}.
+ * After a launch of the shared-operand contraction: {1, 1, accumulator tiles of
+ * 128 B rows, rows formed, B rows, 2, 1, 0, operand stages, field stages, 0}.
  * FBS_ERR_ARG for a bad level or job.
  */
 fbs_status fbs_plan_tc_info(const fbs_plan *plan, int level, int which, int32_t *info);

@@ -191,6 +191,8 @@ __global__ void __launch_bounds__(kCThreads, 1) contract_fp32_kernel(
 // share an item's rows (one thread per item and 304 rows, most of them zero,
 // took 40 to 50 us of dependent loads for any size).  Every sum has a fixed
 // order.  Field blockIdx.y of a batch: partials sfs, outputs ofs further on.
+// NORM (a plan of one level, whose items are the plan's): the estimates too,
+// which saves a launch of 6 us that waits for this one.
 struct ReduceSeg {
     const double *part;
     const int *map;
@@ -198,6 +200,44 @@ struct ReduceSeg {
     int n, ld, rows;
     long long sfs, ofs;
 };
+// The estimates of a sum over the whole plan (NormArgs):
+// B = V^2/N_pix^3 num/(N_pix N_tri), P = V/N_pix^2 sumsq/(N_pix |S_b|)
+// (NaN for empty shells), T = V^3/N_pix^4 qnum/(N_pix N_quad).
+struct NormArgs {
+    const int64_t *ntri;
+    const double *nq;
+    const long long *shell;
+    double *B, *P, *T;  // outputs (any may be null)
+    double L;
+    int N, ntrip, nquad, nbins;
+    const int *err;       // this evaluation's wait-timeout code (or null)
+    int *sticky, *h_err;  // kept until the host reports it, and its pinned host copy
+};
+__device__ __forceinline__ double norm_B(const NormArgs &a, double num, int i) {
+    const double V = a.L * a.L * a.L, npix = (double)a.N * a.N * a.N, cB = V * V / (npix * npix * npix);
+    return cB * num / (npix * (double)a.ntri[i]);
+}
+__device__ __forceinline__ double norm_P(const NormArgs &a, double sumsq, int b) {
+    const double V = a.L * a.L * a.L, npix = (double)a.N * a.N * a.N, cP = V / (npix * npix);
+    return a.shell[b] > 0 ? cP * sumsq / (npix * (double)a.shell[b]) : nan("");
+}
+__device__ __forceinline__ double norm_T(const NormArgs &a, double num, int i) {
+    const double V = a.L * a.L * a.L, npix = (double)a.N * a.N * a.N;
+    const double cT = V * V * V / (npix * npix * npix * npix);
+    return cT * num / (npix * a.nq[i]);
+}
+// A tensor-core wait gave up: the sums are incomplete.  One thread of the
+// grid (`one`) keeps the code and copies it to the host.
+__device__ __forceinline__ bool norm_bad(const NormArgs &a, bool one) {
+    const bool bad = a.err && *a.err;
+    if (one && a.sticky) {
+        const int v = bad ? *a.err : *a.sticky;
+        if (bad) *a.sticky = v;
+        if (a.h_err) *(volatile int *)a.h_err = v;
+    }
+    return bad;
+}
+
 struct ReduceArgs {
     ReduceSeg seg[2];
     int nblk[2];
@@ -207,12 +247,22 @@ struct ReduceArgs {
     int sqrows;
     long long sfs, ofs;
     double scale;
+    NormArgs norm;
 };
 
+template <bool NORM>
 __global__ void __launch_bounds__(256) level_reduce_kernel(const __grid_constant__ ReduceArgs a) {
     __shared__ double red[256];
     const int tid = threadIdx.x;
     int blk = blockIdx.x;
+    const long long f = blockIdx.y;
+    bool bad = false;
+    if (NORM) {
+        bad = norm_bad(a.norm, blk == 0 && f == 0 && tid == 0);
+        if (blk == 0 && a.norm.P)
+            for (int b = tid; b < a.norm.nbins; b += 256)
+                if (a.norm.shell[b] <= 0) a.norm.P[f * a.norm.nbins + b] = nan("");
+    }
     const int which = blk < a.nblk[0] ? 0 : blk < a.nblk[0] + a.nblk[1] ? 1 : 2;
     if (which < 2) {
         const ReduceSeg &g = a.seg[which];
@@ -228,7 +278,11 @@ __global__ void __launch_bounds__(256) level_reduce_kernel(const __grid_constant
         __syncthreads();
         if (ty == 0 && i < g.n) {
             for (int k = 1; k < 8; ++k) s += red[tid + 32 * k];
-            g.out[blockIdx.y * g.ofs + (g.map ? g.map[i] : i)] = a.scale * s;
+            const int o = g.map ? g.map[i] : i;
+            s *= a.scale;
+            g.out[blockIdx.y * g.ofs + o] = s;
+            if (NORM && !which && a.norm.B) a.norm.B[f * a.norm.ntrip + o] = bad ? nan("") : norm_B(a.norm, s, o);
+            if (NORM && which && a.norm.T) a.norm.T[o] = bad ? nan("") : norm_T(a.norm, s, o);
         }
         return;
     }
@@ -244,36 +298,25 @@ __global__ void __launch_bounds__(256) level_reduce_kernel(const __grid_constant
         if (tid < w) red[tid] += red[tid + w];
         __syncthreads();
     }
-    if (tid == 0) a.sumsq[blockIdx.y * a.ofs + a.pbin[blk]] = a.scale * red[0];
+    if (tid == 0) {
+        const int b = a.pbin[blk];
+        s = a.scale * red[0];
+        a.sumsq[blockIdx.y * a.ofs + b] = s;
+        if (NORM && a.norm.P) a.norm.P[f * a.norm.nbins + b] = norm_P(a.norm, s, b);
+    }
 }
 
 // ------------------------------------------------------------------ normalise
-// B = V^2/N_pix^3 num/(N_pix N_tri), P = V/N_pix^2 sumsq/(N_pix |S_b|)
-// (NaN for empty shells), T = V^3/N_pix^4 qnum/(N_pix N_quad).
-__global__ void normalise_kernel(const double *__restrict__ tnum, const int64_t *__restrict__ ntri,
-                                 int ntrip, const double *__restrict__ qnum,
-                                 const double *__restrict__ nq, int nquad,
-                                 const double *__restrict__ sumsq, const long long *__restrict__ shell,
-                                 int nbins, double L, int N, double *__restrict__ B,
-                                 double *__restrict__ P, double *__restrict__ T,
-                                 const int *__restrict__ err, int *__restrict__ sticky) {
-    // field blockIdx.y of a batch: its sums and outputs follow the previous fields'
+// Estimates of a plan of several levels, after the last level's reduction.
+// Field blockIdx.y of a batch: its sums and outputs follow the previous fields'.
+__global__ void normalise_kernel(const __grid_constant__ NormArgs a, const double *__restrict__ tnum,
+                                 const double *__restrict__ qnum, const double *__restrict__ sumsq) {
     const long long f = blockIdx.y;
-    tnum += f * ntrip;
-    sumsq += f * nbins;
-    if (B) B += f * ntrip;
-    if (P) P += f * nbins;
-    const double V = L * L * L;
-    const double npix = (double)N * N * N;
-    const double cB = V * V / (npix * npix * npix);
-    const double cP = V / (npix * npix);
-    const double cT = V * V * V / (npix * npix * npix * npix);
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool bad = err && *err;  // a tensor-core wait gave up: the sums are incomplete
-    if (bad && sticky && i == 0) *sticky = *err;  // kept until the host reports it
-    if (B && i < ntrip) B[i] = bad ? nan("") : cB * tnum[i] / (npix * (double)ntri[i]);
-    if (P && i < nbins) P[i] = shell[i] > 0 ? cP * sumsq[i] / (npix * (double)shell[i]) : nan("");
-    if (T && i < nquad) T[i] = bad ? nan("") : cT * qnum[i] / (npix * nq[i]);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool bad = norm_bad(a, i == 0 && f == 0);
+    if (a.B && i < a.ntrip) a.B[f * a.ntrip + i] = bad ? nan("") : norm_B(a, tnum[f * a.ntrip + i], i);
+    if (a.P && i < a.nbins) a.P[f * a.nbins + i] = norm_P(a, sumsq[f * a.nbins + i], i);
+    if (a.T && i < a.nquad) a.T[i] = bad ? nan("") : norm_T(a, qnum[i], i);
 }
 
 // ------------------------------------------------------------------ connected trispectrum
@@ -698,13 +741,21 @@ void launch_contract_fp32(Plan &p, const float *islab, long long npts, long long
 void launch_level_reduce(Plan &p, bool quads) {
     Plan &R = p.root();
     launch_level_reduce_batch(p, quads, 1, p.fused_active ? p.d_fpart : p.d_tpart, p.d_sumsq_part, R.d_tnum,
-                              R.d_sumsq);
+                              R.d_sumsq, R.d_B, R.d_P);
+}
+
+static NormArgs norm_args(Plan &p, bool quads, double *B, double *P) {
+    const bool tc = p.precision != FBS_PREC_FP32;
+    return NormArgs{p.d_ntri, p.d_nquad, p.d_shell, B, P, quads ? p.d_T : nullptr, p.L, p.N, (int)p.ntri.size(),
+                    quads ? (int)p.nquad.size() : 0, p.nbins, tc ? tc_error_flag(p) : nullptr,
+                    tc ? tc_sticky_flag(p) : nullptr, p.h_err};
 }
 
 // The sums of nf fields (partials tpart: per field part_blocks rows; sumsq
-// partials: per field nbins blocks) into tnum[nf][ntrip], sumsq[nf][nbins].
+// partials: per field nbins blocks) into tnum[nf][ntrip], sumsq[nf][nbins];
+// the estimates of a plan of one level too.
 void launch_level_reduce_batch(Plan &p, bool quads, int nf, const double *tpart, const double *sq,
-                               double *tnum, double *sumsq) {
+                               double *tnum, double *sumsq, double *B, double *P) {
     Plan &R = p.root();
     KTimer tm(p, KC_REDUCE);
     const double r = (double)R.N / (double)p.M;
@@ -724,27 +775,30 @@ void launch_level_reduce_batch(Plan &p, bool quads, int nf, const double *tpart,
     a.sqrows = p.M * zstage_row_groups(p.M);
     a.sfs = (long long)p.nbins * a.sqrows;
     a.ofs = R.nbins;
-    level_reduce_kernel<<<dim3(a.nblk[0] + a.nblk[1] + p.nbins, nf), 256, 0, p.stream>>>(a);
+    const dim3 grid(a.nblk[0] + a.nblk[1] + p.nbins, nf);
+    if (R.levels.size() == 1) {
+        a.norm = norm_args(R, quads, B, P);
+        level_reduce_kernel<true><<<grid, 256, 0, p.stream>>>(a);
+    } else {
+        level_reduce_kernel<false><<<grid, 256, 0, p.stream>>>(a);
+    }
     FBS_CUDA(cudaGetLastError());
 }
 
 void launch_normalise(Plan &p, bool quads) { launch_normalise_batch(p, quads, 1, p.d_tnum, p.d_sumsq, p.d_B, p.d_P); }
 
-// B[nf][ntrip], P[nf][nbins] from tnum[nf][ntrip], sumsq[nf][nbins]; T (single field only).
+// B[nf][ntrip], P[nf][nbins] from tnum[nf][ntrip], sumsq[nf][nbins]; T (single
+// field only).  A plan of one level has them from its reduction.
 void launch_normalise_batch(Plan &p, bool quads, int nf, const double *tnum, const double *sumsq, double *B,
                             double *P) {
-    KTimer tm(p, KC_REDUCE);
-    int ntrip = (int)p.ntri.size(), nquad = quads ? (int)p.nquad.size() : 0;
-    int n_all = std::max(std::max(ntrip, nquad), p.nbins);
-    dim3 grid((n_all + 255) / 256, nf);
-    normalise_kernel<<<grid, 256, 0, p.stream>>>(
-        tnum, p.d_ntri, ntrip, p.d_qnum, p.d_nquad, nquad, sumsq, p.d_shell, p.nbins,
-        p.L, p.N, B, P, quads ? p.d_T : nullptr,
-        p.precision != FBS_PREC_FP32 ? tc_error_flag(p) : nullptr,
-        p.precision != FBS_PREC_FP32 ? tc_sticky_flag(p) : nullptr);
-    FBS_CUDA(cudaGetLastError());
+    if (p.levels.size() != 1) {
+        KTimer tm(p, KC_REDUCE);
+        const NormArgs a = norm_args(p, quads, B, P);
+        const int n_all = std::max(std::max(a.ntrip, a.nquad), a.nbins);
+        normalise_kernel<<<dim3((n_all + 255) / 256, nf), 256, 0, p.stream>>>(a, tnum, p.d_qnum, sumsq);
+        FBS_CUDA(cudaGetLastError());
+    }
     if (p.precision != FBS_PREC_FP32 && tc_sticky_flag(p) && p.h_err) {
-        FBS_CUDA(cudaMemcpyAsync(p.h_err, tc_sticky_flag(p), sizeof(int), cudaMemcpyDeviceToHost, p.stream));
         FBS_CUDA(cudaEventRecord(p.ev_err, p.stream));
         p.err_recorded = true;
     }
@@ -775,7 +829,7 @@ void launch_count_contraction(Plan &p, const double *noct, int nbins_all, int, c
     a.scale = 1.0;
     a.seg[0] = ReduceSeg{part, nullptr, d_den, nitems, nitems, blocks, 0, 0};
     a.nblk[0] = (nitems + 31) / 32;
-    level_reduce_kernel<<<a.nblk[0], 256, 0, p.stream>>>(a);
+    level_reduce_kernel<false><<<a.nblk[0], 256, 0, p.stream>>>(a);
     FBS_CUDA(cudaGetLastError());
 }
 

@@ -135,8 +135,8 @@ void launch_forward(Plan &p, const float *d_field, const float *const *d_fields,
 void launch_forward_grid(Plan &p, int N, const BoxGeom &bx, const FftFactors &fN, const float2 *tw,
                          const float *d_field, const float *const *d_fields, int nf, float2 *zbuf, float2 *ybuf,
                          float2 *box, const FieldPairs *pairs = nullptr);
-void launch_inverse_x(Plan &p, bool indicator_fp64);
-void launch_inverse_x_geom(Plan &p, const BinGeom *geom, int nb, int nvb);
+void launch_inverse_x(Plan &p, int *clear = nullptr);
+void launch_inverse_x_geom(Plan &p, const BinGeom *geom, int nb, int nvb, int *clear = nullptr);
 void launch_inverse_yz_slab(Plan &p, int x0, int nx, float *islab);
 void launch_inverse_yz_slab_geom(Plan &p, int x0, int nx, float *islab, const BinGeom *geom, int nb, int nvb,
                                  double *sq);
@@ -182,12 +182,12 @@ bool gram_job_info(Plan &p, bool fused, int32_t *out);
 void free_gram_state(Plan &p);
 void launch_level_reduce(Plan &level, bool quads);
 void launch_level_reduce_batch(Plan &level, bool quads, int nf, const double *tpart, const double *sq,
-                               double *tnum, double *sumsq);
+                               double *tnum, double *sumsq, double *B, double *P);
 void launch_normalise(Plan &root, bool quads);
 void launch_normalise_batch(Plan &root, bool quads, int nf, const double *tnum, const double *sumsq, double *B,
                             double *P);
-// Connected trispectrum of the last evaluation into d_Tc[nquad] (root).
 constexpr int kMomChunks = 64;  // partials per bin of the shell moments
+// Connected trispectrum of the last evaluation into d_Tc[nquad] (root).
 void launch_connected(Plan &root, double *d_Tc);
 std::vector<int> fast_grids();  // grids with compile-time-radix kernels for every inverse stage
 void prepare_fp32(Plan &level, bool trip, bool quads);
@@ -265,7 +265,7 @@ struct Plan {
     // device memory
     std::vector<void *> allocs;
     long long dev_bytes = 0;
-    // timeout reporting: the normalisation copies the device's sticky flag
+    // timeout reporting: the normalisation writes the device's sticky flag
     // into h_err (pinned) at the end of every tensor-core evaluation and
     // records ev_err, so later calls can see a timeout without waiting
     int *h_err = nullptr;

@@ -180,7 +180,9 @@ __global__ void __launch_bounds__(kThreads) inv_x_kernel(const float2 *__restric
                                                          typename V2<T>::t *__restrict__ A, int nl,
                                                          FftFactors f,
                                                          const typename V2<T>::t *__restrict__ tw,
-                                                         const double *__restrict__ wtab = nullptr) {
+                                                         const double *__restrict__ wtab = nullptr,
+                                                         int *__restrict__ clear = nullptr) {
+    if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
     typedef typename V2<T>::t C;
     extern __shared__ __align__(16) unsigned char smraw[];
     C *a = reinterpret_cast<C *>(smraw);
@@ -889,9 +891,11 @@ __global__ void __launch_bounds__(T *LP) fwd_z_reg_kernel(const float *__restric
 template <int N, int N1, int N2, int T, int LP>
 __global__ void __launch_bounds__(T *LP) inv_x_reg_kernel(const float2 *__restrict__ box, BoxGeom bg,
                                                           const BinGeom *__restrict__ geom,
-                                                          float2 *__restrict__ A, const float2 *__restrict__ tw) {
+                                                          float2 *__restrict__ A, const float2 *__restrict__ tw,
+                                                          int *__restrict__ clear) {
     static_assert(N1 * N2 == N && N1 % T == 0 && N2 % T == 0, "threads must divide both passes");
     __shared__ float2 tile[N * LP];
+    if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
     const BinGeom g = geom[blockIdx.y];
     if (g.empty) return;
     const int ngz = (g.Dzb + LP - 1) / LP;
@@ -1206,11 +1210,12 @@ static int max_dzb(const Plan &p, int bin0, int nb) {
     return m;
 }
 
-void launch_inverse_x(Plan &p, bool) { launch_inverse_x_geom(p, p.d_geom, p.nbins, p.nbins); }
+void launch_inverse_x(Plan &p, int *clear) { launch_inverse_x_geom(p, p.d_geom, p.nbins, p.nbins, clear); }
 
 // x stage over `nvb` (virtual) bins of geometry table `geom`; bins i and
-// i mod nb share their extents (batched fields repeat the level's bins).
-void launch_inverse_x_geom(Plan &p, const BinGeom *geom, int nb, int nvb) {
+// i mod nb share their extents (batched fields repeat the level's bins).  The
+// first level's x stage zeroes the evaluation's timeout flag, `clear`.
+void launch_inverse_x_geom(Plan &p, const BinGeom *geom, int nb, int nvb, int *clear) {
     const int N = p.M;  // inverse transforms run on the evaluation grid
     const int nl = lines_per_cta<float>(N);
     const size_t sm = 2 * (size_t)nl * (N + 1) * sizeof(float2);
@@ -1226,7 +1231,7 @@ void launch_inverse_x_geom(Plan &p, const BinGeom *geom, int nb, int nvb) {
         dim3 grid(gx, nvb);
 #define FBS_XR(n, n1, n2, t_, lp_)                                                    \
     if (N == n) inv_x_reg_kernel<n, n1, n2, t_, lp_><<<grid, t_ * lp_, 0, p.stream>>>( \
-                    p.d_box, p.boxM, geom, p.d_A, p.d_twM);
+                    p.d_box, p.boxM, geom, p.d_A, p.d_twM, clear);
         FBS_YREG_LIST(FBS_XR)
 #undef FBS_XR
         FBS_CUDA(cudaGetLastError());
@@ -1239,7 +1244,7 @@ void launch_inverse_x_geom(Plan &p, const BinGeom *geom, int nb, int nvb) {
 #undef FBS_PICK
     allow_smem(k, sm);
     dim3 grid(max_inv_x_grid(p, 0, nb, nl), nvb);
-    k<<<grid, kThreads, sm, p.stream>>>(p.d_box, p.boxM, geom, 0, p.d_A, nl, p.fM, p.d_twM, nullptr);
+    k<<<grid, kThreads, sm, p.stream>>>(p.d_box, p.boxM, geom, 0, p.d_A, nl, p.fM, p.d_twM, nullptr, clear);
     FBS_CUDA(cudaGetLastError());
 }
 
@@ -1333,7 +1338,7 @@ void launch_count_fields_fp64_impl(Plan &p, double *noct, int bin0, int nb, doub
         auto k = inv_x_kernel<double, true>;
         allow_smem(k, sm);
         dim3 grid(max_inv_x_grid(p, bin0, nb, nl), nb);
-        k<<<grid, kThreads, sm, p.stream>>>(p.d_box, p.boxM, d_geom_grp, 0, A64, nl, p.fM, p.d_tw64, wtab);
+        k<<<grid, kThreads, sm, p.stream>>>(p.d_box, p.boxM, d_geom_grp, 0, A64, nl, p.fM, p.d_tw64, wtab, nullptr);
         FBS_CUDA(cudaGetLastError());
     }
     {

@@ -972,13 +972,12 @@ static void forward_or_follow(Plan &p, const float *field) {
 // 2e-5 within which a caller may rely on repeated results.
 static void run_field(Plan &p, const float *field, bool quads, bool connected = false) {
     const bool tc = p.precision != FBS_PREC_FP32;
-    if (tc) FBS_CUDA(cudaMemsetAsync(p.d_errbuf, 0, sizeof(int), p.stream));
     forward_or_follow(p, field);
     for (Plan *lp : p.levels) {
         Plan &lv = *lp;
         lv.gram_off = connected;
         lv.fused_active = quads && tc && tc_fused_usable(lv);
-        launch_inverse_x(lv, false);
+        launch_inverse_x(lv, tc && lp == p.levels[0] ? p.d_errbuf : nullptr);
         const int M = lv.M;
         const long long plane = (long long)M * M;
         for (int s = 0; s < lv.nslabs; ++s) {
@@ -1106,7 +1105,6 @@ static void run_batch(Plan &p, const float *const *fields, int nf) {
         bs.ptrs = ptrs;
     }
     const bool tc = p.precision != FBS_PREC_FP32;
-    if (tc) FBS_CUDA(cudaMemsetAsync(p.d_errbuf, 0, sizeof(int), p.stream));
     launch_forward(p, nullptr, bs.d_fptrs, nf, bs.zbuf, bs.ybuf, bs.box);
     for (size_t l = 0; l < p.levels.size(); ++l) {
         Plan &lv = *p.levels[l];
@@ -1124,7 +1122,7 @@ static void run_batch(Plan &p, const float *const *fields, int nf) {
         lv.gram_off = false;
         try {
             const int M = lv.M, nb = lv.nbins;
-            launch_inverse_x_geom(lv, bl.d_vgeom, nb, nf * nb);
+            launch_inverse_x_geom(lv, bl.d_vgeom, nb, nf * nb, tc && l == 0 ? p.d_errbuf : nullptr);
             const long long plane = (long long)M * M;
             for (int s = 0; s < bl.nslabs; ++s) {
                 const int x0 = s * bl.slab;
@@ -1138,7 +1136,7 @@ static void run_batch(Plan &p, const float *const *fields, int nf) {
                 else
                     launch_contract_fp32(lv, bs.I, npts, stride, false, nf, bl.tpart);
             }
-            launch_level_reduce_batch(lv, false, nf, bl.tpart, bl.sq, bs.tnum, bs.sumsq);
+            launch_level_reduce_batch(lv, false, nf, bl.tpart, bl.sq, bs.tnum, bs.sumsq, bs.B, bs.P);
         } catch (...) {
             lv.d_A = A0;
             lv.d_G = G0;
@@ -1316,7 +1314,7 @@ static void run_diagonal(Plan &p, const float *field) {
         lv.d_G = Gfull.as<float2>();
         lv.slab = M;
         try {
-            launch_inverse_x(lv, false);
+            launch_inverse_x(lv);
             launch_inverse_yz_slab_geom(lv, 0, M, Ifull.as<float>(), dl.d_geom_full, nb, nb, sq.as<double>());
         } catch (...) {
             lv.d_G = G0;
