@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "chain.cuh"
 #include "fbs_internal.h"
 #include "fft_core.cuh"
 
@@ -72,6 +73,7 @@ __global__ void __launch_bounds__(kThreads) fwd_z_kernel(const float *__restrict
                                                          float2 *__restrict__ zbuf_all, long long zstride,
                                                          int N, int Dz, int nl, FftFactors f,
                                                          const float2 *__restrict__ tw) {
+    chain_begin();
     const float *__restrict__ field = PROD ? fp.base + fp.pairs[blockIdx.y].x * fp.stride
                                            : fields ? fields[blockIdx.y] : field_one;
     const float *__restrict__ other = PROD ? fp.base + fp.pairs[blockIdx.y].y * fp.stride : nullptr;
@@ -114,6 +116,7 @@ __global__ void __launch_bounds__(kThreads) fwd_y_kernel(const float2 *__restric
                                                          float2 *__restrict__ ybuf_all, long long zstride,
                                                          long long ystride, int N, int D, int Dz, int nl,
                                                          FftFactors f, const float2 *__restrict__ tw) {
+    chain_begin();
     const float2 *__restrict__ zbuf = zbuf_all + (long long)blockIdx.z * zstride;  // field blockIdx.z
     float2 *__restrict__ ybuf = ybuf_all + (long long)blockIdx.z * ystride;
     extern __shared__ float2 sm[];
@@ -145,6 +148,7 @@ __global__ void __launch_bounds__(kThreads) fwd_x_kernel(const float2 *__restric
                                                          float2 *__restrict__ box_all, long long ystride,
                                                          long long bstride, int N, int D, int Dz, int nl,
                                                          FftFactors f, const float2 *__restrict__ tw) {
+    chain_begin();
     const float2 *__restrict__ ybuf = ybuf_all + (long long)blockIdx.z * ystride;  // field blockIdx.z
     float2 *__restrict__ box = box_all + (long long)blockIdx.z * bstride;
     extern __shared__ float2 sm[];
@@ -182,6 +186,7 @@ __global__ void __launch_bounds__(kThreads) inv_x_kernel(const float2 *__restric
                                                          const typename V2<T>::t *__restrict__ tw,
                                                          const double *__restrict__ wtab = nullptr,
                                                          int *__restrict__ clear = nullptr) {
+    chain_begin();
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
     typedef typename V2<T>::t C;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -239,6 +244,7 @@ __global__ void __launch_bounds__(kThreads) inv_y_kernel(const typename V2<T>::t
                                                          long long G_stride_plane_unused, int nl,
                                                          FftFactors f,
                                                          const typename V2<T>::t *__restrict__ tw) {
+    chain_begin();
     typedef typename V2<T>::t C;
     extern __shared__ __align__(16) unsigned char smraw[];
     C *a = reinterpret_cast<C *>(smraw);
@@ -290,6 +296,7 @@ __global__ void __launch_bounds__(kThreads) inv_z_kernel(const typename V2<T>::t
                                                          double *__restrict__ sumsq_part, int nl,
                                                          FftFactors f,
                                                          const typename V2<T>::t *__restrict__ tw) {
+    chain_begin();
     typedef typename V2<T>::t C;
     extern __shared__ __align__(16) unsigned char smraw[];
     C *a = reinterpret_cast<C *>(smraw);
@@ -435,6 +442,7 @@ __global__ void __launch_bounds__(T *LP) inv_z_fast_kernel(const float2 *__restr
                                                            long long out_bin_stride,
                                                            double *__restrict__ sumsq_part,
                                                            const float2 *__restrict__ tw) {
+    chain_begin();
     static_assert(R0 * R1 * R2 * R3 == N, "radices must multiply to N");
     // line stride: padded line, rounded to 8 mod 16 slots so that the two
     // lines a warp spans (T = 16) sit on opposite halves of the banks
@@ -627,6 +635,7 @@ __global__ void __launch_bounds__(T *LP) inv_z_reg_kernel(const float2 *__restri
                                                           long long out_bin_stride,
                                                           double *__restrict__ sumsq_part,
                                                           const float2 *__restrict__ tw) {
+    chain_begin();
     static_assert(N1 * N2 == N && N1 % T == 0 && N2 % T == 0, "threads must divide both passes");
     static_assert((T * LP) % 32 == 0, "whole warps");
     // tile row padded by one slot (conflict-free column reads in pass B); line
@@ -747,6 +756,7 @@ template <int N, int N1, int N2, int T, int LP>
 __global__ void __launch_bounds__(T *LP) inv_y_reg_kernel(const float2 *__restrict__ A,
                                                           const BinGeom *__restrict__ geom, int x0,
                                                           float2 *__restrict__ G, const float2 *__restrict__ tw) {
+    chain_begin();
     static_assert(N1 * N2 == N && N1 % T == 0 && N2 % T == 0, "threads must divide both passes");
     __shared__ float2 tile[N * LP];
     const BinGeom g = geom[blockIdx.z];
@@ -812,6 +822,7 @@ __global__ void __launch_bounds__(T *LP) fwd_z_reg_kernel(const float *__restric
                                                           const float *const *__restrict__ fields, FieldPairs fp,
                                                           float2 *__restrict__ zbuf_all, long long zstride, int Dz,
                                                           const float2 *__restrict__ tw) {
+    chain_begin();
     static_assert(N1 * N2 == N && N1 % T == 0 && N2 % T == 0, "threads must divide both passes");
     static_assert((T * LP) % 32 == 0, "whole warps");
     constexpr int LD = N1 + 1;
@@ -893,6 +904,7 @@ __global__ void __launch_bounds__(T *LP) inv_x_reg_kernel(const float2 *__restri
                                                           const BinGeom *__restrict__ geom,
                                                           float2 *__restrict__ A, const float2 *__restrict__ tw,
                                                           int *__restrict__ clear) {
+    chain_begin();
     static_assert(N1 * N2 == N && N1 % T == 0 && N2 % T == 0, "threads must divide both passes");
     __shared__ float2 tile[N * LP];
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
@@ -1139,6 +1151,7 @@ void launch_forward_grid(Plan &p, int N, const BoxGeom &bx, const FftFactors &fN
     const FieldPairs fp = pairs ? *pairs : FieldPairs{nullptr, 0, nullptr};
     const int D = bx.D, Dz = bx.Dz;
     const long long zs = (long long)N * N * Dz, ys = (long long)N * D * Dz, bs = (long long)D * D * Dz;
+    const bool chained = (long long)nf * N * N * N <= kChainValues / 4;
     const int nl = lines_per_cta<float>(N);
     const size_t sm = 2 * (size_t)nl * (N + 1) * sizeof(float2);
     auto kz = pairs ? fwd_z_kernel<true> : fwd_z_kernel<false>;
@@ -1181,14 +1194,14 @@ void launch_forward_grid(Plan &p, int N, const BoxGeom &bx, const FftFactors &fN
         KTimer t(p, KC_FWD_Y);
         allow_smem(ky, sm);
         dim3 grid((Dz + nl - 1) / nl, N, nf);
-        ky<<<grid, kThreads, sm, p.stream>>>(zbuf, ybuf, zs, ys, N, D, Dz, nl, fN, tw);
+        launch_chained(chained, ky, grid, kThreads, sm, p.stream, zbuf, ybuf, zs, ys, N, D, Dz, nl, fN, tw);
         FBS_CUDA(cudaGetLastError());
     }
     {
         KTimer t(p, KC_FWD_X);
         allow_smem(kx, sm);
         dim3 grid((Dz + nl - 1) / nl, D, nf);
-        kx<<<grid, kThreads, sm, p.stream>>>(ybuf, box, ys, bs, N, D, Dz, nl, fN, tw);
+        launch_chained(chained, kx, grid, kThreads, sm, p.stream, ybuf, box, ys, bs, N, D, Dz, nl, fN, tw);
         FBS_CUDA(cudaGetLastError());
     }
 }
@@ -1217,6 +1230,7 @@ void launch_inverse_x(Plan &p, int *clear) { launch_inverse_x_geom(p, p.d_geom, 
 // first level's x stage zeroes the evaluation's timeout flag, `clear`.
 void launch_inverse_x_geom(Plan &p, const BinGeom *geom, int nb, int nvb, int *clear) {
     const int N = p.M;  // inverse transforms run on the evaluation grid
+    const bool chained = (long long)nvb * N * N * N <= kChainValues;
     const int nl = lines_per_cta<float>(N);
     const size_t sm = 2 * (size_t)nl * (N + 1) * sizeof(float2);
     KTimer t(p, KC_INV_X);
@@ -1230,8 +1244,9 @@ void launch_inverse_x_geom(Plan &p, const BinGeom *geom, int nb, int nvb, int *c
             if (!p.geom[b].empty) gx = std::max(gx, p.geom[b].Db * ((p.geom[b].Dzb + lp - 1) / lp));
         dim3 grid(gx, nvb);
 #define FBS_XR(n, n1, n2, t_, lp_)                                                    \
-    if (N == n) inv_x_reg_kernel<n, n1, n2, t_, lp_><<<grid, t_ * lp_, 0, p.stream>>>( \
-                    p.d_box, p.boxM, geom, p.d_A, p.d_twM, clear);
+    if (N == n)                                                                       \
+        launch_chained(chained, inv_x_reg_kernel<n, n1, n2, t_, lp_>, grid, t_ * lp_, 0, p.stream, p.d_box, p.boxM, geom, \
+                       p.d_A, p.d_twM, clear);
         FBS_YREG_LIST(FBS_XR)
 #undef FBS_XR
         FBS_CUDA(cudaGetLastError());
@@ -1244,7 +1259,7 @@ void launch_inverse_x_geom(Plan &p, const BinGeom *geom, int nb, int nvb, int *c
 #undef FBS_PICK
     allow_smem(k, sm);
     dim3 grid(max_inv_x_grid(p, 0, nb, nl), nvb);
-    k<<<grid, kThreads, sm, p.stream>>>(p.d_box, p.boxM, geom, 0, p.d_A, nl, p.fM, p.d_twM, nullptr, clear);
+    launch_chained(chained, k, grid, kThreads, sm, p.stream, p.d_box, p.boxM, geom, 0, p.d_A, nl, p.fM, p.d_twM, nullptr, clear);
     FBS_CUDA(cudaGetLastError());
 }
 
@@ -1257,6 +1272,7 @@ void launch_inverse_yz_slab(Plan &p, int x0, int nx, float *islab) {
 void launch_inverse_yz_slab_geom(Plan &p, int x0, int nx, float *islab, const BinGeom *geom, int nb, int nvb,
                                  double *sq) {
     const int N = p.M;  // evaluation grid
+    const bool chained = (long long)nvb * N * N * N <= kChainValues;
     const int nl = lines_per_cta<float>(N);
     const size_t sm = 2 * (size_t)nl * (N + 1) * sizeof(float2);
     static const char *yenv = getenv("FBS_YSTAGE");
@@ -1266,8 +1282,9 @@ void launch_inverse_yz_slab_geom(Plan &p, int x0, int nx, float *islab, const Bi
         const int lp = yreg_lines(N);
         dim3 grid((max_dzb(p, 0, nb) + lp - 1) / lp, nx, nvb);
 #define FBS_YR(n, n1, n2, t, lp_)                                                        \
-    if (N == n) inv_y_reg_kernel<n, n1, n2, t, lp_><<<grid, t * lp_, 0, p.stream>>>(      \
-                    p.d_A, geom, x0, p.d_G, p.d_twM);
+    if (N == n)                                                                          \
+        launch_chained(chained, inv_y_reg_kernel<n, n1, n2, t, lp_>, grid, t * lp_, 0, p.stream, p.d_A, geom, x0, p.d_G, \
+                       p.d_twM);
         FBS_YREG_LIST(FBS_YR)
 #undef FBS_YR
         FBS_CUDA(cudaGetLastError());
@@ -1282,7 +1299,7 @@ void launch_inverse_yz_slab_geom(Plan &p, int x0, int nx, float *islab, const Bi
         if (getenv("FBS_GENERIC_Y")) k = inv_y_kernel<float>;
         allow_smem(k, sm);
         dim3 grid((max_dzb(p, 0, nb) + nl - 1) / nl, nx, nvb);
-        k<<<grid, kThreads, sm, p.stream>>>(p.d_A, geom, 0, N, x0, p.d_G, 0, nl, p.fM, p.d_twM);
+        launch_chained(chained, k, grid, kThreads, sm, p.stream, p.d_A, geom, 0, N, x0, p.d_G, 0, nl, p.fM, p.d_twM);
         FBS_CUDA(cudaGetLastError());
     }
     const int zk = zstage_kind(N);
@@ -1296,7 +1313,7 @@ void launch_inverse_yz_slab_geom(Plan &p, int x0, int nx, float *islab, const Bi
         auto k = inv_z_reg_kernel<n, n1, n2, t, lp>;                                                        \
         const size_t dyn = (size_t)2 * lp * dz * sizeof(float2);                                            \
         const int G = std::min(nitems, resident_ctas(k, t * lp, dyn));                                      \
-        k<<<G, t * lp, dyn, p.stream>>>(p.d_G, geom, x0, nx, nitems, islab, obs, sq, p.d_twM);              \
+        launch_chained(chained, k, G, t * lp, dyn, p.stream, p.d_G, geom, x0, nx, nitems, islab, obs, sq, p.d_twM);   \
     }
         FBS_ZREG_LIST(FBS_ZR)
 #undef FBS_ZR
@@ -1307,7 +1324,7 @@ void launch_inverse_yz_slab_geom(Plan &p, int x0, int nx, float *islab, const Bi
         const long long obs = (long long)p.slab * N * N;
 #define FBS_ZL(n, t, lp, a, b, c, d)                                                          \
     if (N == n)                                                                               \
-        inv_z_fast_kernel<n, t, lp, a, b, c, d><<<grid, t * lp, 0, p.stream>>>(                \
+        launch_chained(chained, inv_z_fast_kernel<n, t, lp, a, b, c, d>, grid, t * lp, 0, p.stream,    \
             p.d_G, geom, x0, islab, obs, sq, p.d_twM);
         FBS_ZFAST_LIST(FBS_ZL)
 #undef FBS_ZL
@@ -1317,7 +1334,7 @@ void launch_inverse_yz_slab_geom(Plan &p, int x0, int nx, float *islab, const Bi
         auto k = inv_z_kernel<float, false>;
         allow_smem(k, sm);
         dim3 grid((N + 2 * nl - 1) / (2 * nl), nx, nvb);
-        k<<<grid, kThreads, sm, p.stream>>>(p.d_G, geom, 0, N, x0, islab,
+        launch_chained(chained, k, grid, kThreads, sm, p.stream, p.d_G, geom, 0, N, x0, islab,
                                             (long long)p.slab * N * N, sq, nl, p.fM,
                                             p.d_twM);
         FBS_CUDA(cudaGetLastError());
