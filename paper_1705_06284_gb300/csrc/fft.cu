@@ -72,8 +72,8 @@ __global__ void __launch_bounds__(kThreads) fwd_z_kernel(const float *__restrict
                                                          const float *const *__restrict__ fields, FieldPairs fp,
                                                          float2 *__restrict__ zbuf_all, long long zstride,
                                                          int N, int Dz, int nl, FftFactors f,
-                                                         const float2 *__restrict__ tw) {
-    chain_begin();
+                                                         const float2 *__restrict__ tw, int chained) {
+    chain_begin(chained);
     const float *__restrict__ field = PROD ? fp.base + fp.pairs[blockIdx.y].x * fp.stride
                                            : fields ? fields[blockIdx.y] : field_one;
     const float *__restrict__ other = PROD ? fp.base + fp.pairs[blockIdx.y].y * fp.stride : nullptr;
@@ -115,8 +115,8 @@ template <int... Rs>
 __global__ void __launch_bounds__(kThreads) fwd_y_kernel(const float2 *__restrict__ zbuf_all,
                                                          float2 *__restrict__ ybuf_all, long long zstride,
                                                          long long ystride, int N, int D, int Dz, int nl,
-                                                         FftFactors f, const float2 *__restrict__ tw) {
-    chain_begin();
+                                                         FftFactors f, const float2 *__restrict__ tw, int chained) {
+    chain_begin(chained);
     const float2 *__restrict__ zbuf = zbuf_all + (long long)blockIdx.z * zstride;  // field blockIdx.z
     float2 *__restrict__ ybuf = ybuf_all + (long long)blockIdx.z * ystride;
     extern __shared__ float2 sm[];
@@ -147,8 +147,8 @@ template <int... Rs>
 __global__ void __launch_bounds__(kThreads) fwd_x_kernel(const float2 *__restrict__ ybuf_all,
                                                          float2 *__restrict__ box_all, long long ystride,
                                                          long long bstride, int N, int D, int Dz, int nl,
-                                                         FftFactors f, const float2 *__restrict__ tw) {
-    chain_begin();
+                                                         FftFactors f, const float2 *__restrict__ tw, int chained) {
+    chain_begin(chained);
     const float2 *__restrict__ ybuf = ybuf_all + (long long)blockIdx.z * ystride;  // field blockIdx.z
     float2 *__restrict__ box = box_all + (long long)blockIdx.z * bstride;
     extern __shared__ float2 sm[];
@@ -184,9 +184,9 @@ __global__ void __launch_bounds__(kThreads) inv_x_kernel(const float2 *__restric
                                                          typename V2<T>::t *__restrict__ A, int nl,
                                                          FftFactors f,
                                                          const typename V2<T>::t *__restrict__ tw,
-                                                         const double *__restrict__ wtab = nullptr,
-                                                         int *__restrict__ clear = nullptr) {
-    chain_begin();
+                                                         const double *__restrict__ wtab,
+                                                         int *__restrict__ clear, int chained) {
+    chain_begin(chained);
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
     typedef typename V2<T>::t C;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -243,8 +243,8 @@ __global__ void __launch_bounds__(kThreads) inv_y_kernel(const typename V2<T>::t
                                                          typename V2<T>::t *__restrict__ G,
                                                          long long G_stride_plane_unused, int nl,
                                                          FftFactors f,
-                                                         const typename V2<T>::t *__restrict__ tw) {
-    chain_begin();
+                                                         const typename V2<T>::t *__restrict__ tw, int chained) {
+    chain_begin(chained);
     typedef typename V2<T>::t C;
     extern __shared__ __align__(16) unsigned char smraw[];
     C *a = reinterpret_cast<C *>(smraw);
@@ -295,8 +295,8 @@ __global__ void __launch_bounds__(kThreads) inv_z_kernel(const typename V2<T>::t
                                                          long long out_bin_stride,
                                                          double *__restrict__ sumsq_part, int nl,
                                                          FftFactors f,
-                                                         const typename V2<T>::t *__restrict__ tw) {
-    chain_begin();
+                                                         const typename V2<T>::t *__restrict__ tw, int chained) {
+    chain_begin(chained);
     typedef typename V2<T>::t C;
     extern __shared__ __align__(16) unsigned char smraw[];
     C *a = reinterpret_cast<C *>(smraw);
@@ -441,8 +441,8 @@ __global__ void __launch_bounds__(T *LP) inv_z_fast_kernel(const float2 *__restr
                                                            float *__restrict__ out,
                                                            long long out_bin_stride,
                                                            double *__restrict__ sumsq_part,
-                                                           const float2 *__restrict__ tw) {
-    chain_begin();
+                                                           const float2 *__restrict__ tw, int chained) {
+    chain_begin(chained);
     static_assert(R0 * R1 * R2 * R3 == N, "radices must multiply to N");
     // line stride: padded line, rounded to 8 mod 16 slots so that the two
     // lines a warp spans (T = 16) sit on opposite halves of the banks
@@ -634,8 +634,8 @@ __global__ void __launch_bounds__(T *LP) inv_z_reg_kernel(const float2 *__restri
                                                           int nitems, float *__restrict__ out,
                                                           long long out_bin_stride,
                                                           double *__restrict__ sumsq_part,
-                                                          const float2 *__restrict__ tw) {
-    chain_begin();
+                                                          const float2 *__restrict__ tw, int chained) {
+    chain_begin(chained);
     static_assert(N1 * N2 == N && N1 % T == 0 && N2 % T == 0, "threads must divide both passes");
     static_assert((T * LP) % 32 == 0, "whole warps");
     // tile row padded by one slot (conflict-free column reads in pass B); line
@@ -755,8 +755,8 @@ __global__ void __launch_bounds__(T *LP) inv_z_reg_kernel(const float2 *__restri
 template <int N, int N1, int N2, int T, int LP>
 __global__ void __launch_bounds__(T *LP) inv_y_reg_kernel(const float2 *__restrict__ A,
                                                           const BinGeom *__restrict__ geom, int x0,
-                                                          float2 *__restrict__ G, const float2 *__restrict__ tw) {
-    chain_begin();
+                                                          float2 *__restrict__ G, const float2 *__restrict__ tw, int chained) {
+    chain_begin(chained);
     static_assert(N1 * N2 == N && N1 % T == 0 && N2 % T == 0, "threads must divide both passes");
     __shared__ float2 tile[N * LP];
     const BinGeom g = geom[blockIdx.z];
@@ -821,8 +821,8 @@ template <int N, int N1, int N2, int T, int LP, bool PROD>
 __global__ void __launch_bounds__(T *LP) fwd_z_reg_kernel(const float *__restrict__ field_one,
                                                           const float *const *__restrict__ fields, FieldPairs fp,
                                                           float2 *__restrict__ zbuf_all, long long zstride, int Dz,
-                                                          const float2 *__restrict__ tw) {
-    chain_begin();
+                                                          const float2 *__restrict__ tw, int chained) {
+    chain_begin(chained);
     static_assert(N1 * N2 == N && N1 % T == 0 && N2 % T == 0, "threads must divide both passes");
     static_assert((T * LP) % 32 == 0, "whole warps");
     constexpr int LD = N1 + 1;
@@ -903,8 +903,8 @@ template <int N, int N1, int N2, int T, int LP>
 __global__ void __launch_bounds__(T *LP) inv_x_reg_kernel(const float2 *__restrict__ box, BoxGeom bg,
                                                           const BinGeom *__restrict__ geom,
                                                           float2 *__restrict__ A, const float2 *__restrict__ tw,
-                                                          int *__restrict__ clear) {
-    chain_begin();
+                                                          int *__restrict__ clear, int chained) {
+    chain_begin(chained);
     static_assert(N1 * N2 == N && N1 % T == 0 && N2 % T == 0, "threads must divide both passes");
     __shared__ float2 tile[N * LP];
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
@@ -1177,16 +1177,16 @@ void launch_forward_grid(Plan &p, int N, const BoxGeom &bx, const FftFactors &fN
 #define FBS_FZ(n, n1, n2, t_, lp_)                                                                              \
     if (N == n && pairs)                                                                                        \
         fwd_z_reg_kernel<n, n1, n2, t_, lp_, true><<<grid, t_ * lp_, 0, p.stream>>>(nullptr, nullptr, fp, zbuf, \
-                                                                                    zs, Dz, tw);                \
+                                                                                    zs, Dz, tw, chained);       \
     else if (N == n)                                                                                            \
         fwd_z_reg_kernel<n, n1, n2, t_, lp_, false><<<grid, t_ * lp_, 0, p.stream>>>(d_field, d_fields, fp,     \
-                                                                                     zbuf, zs, Dz, tw);
+                                                                                     zbuf, zs, Dz, tw, chained);
             FBS_ZREG_LIST(FBS_FZ)
 #undef FBS_FZ
         } else {
             allow_smem(kz, sm);
             dim3 grid((int)((rows + 2 * nl - 1) / (2 * nl)), nf);
-            kz<<<grid, kThreads, sm, p.stream>>>(d_field, d_fields, fp, zbuf, zs, N, Dz, nl, fN, tw);
+            kz<<<grid, kThreads, sm, p.stream>>>(d_field, d_fields, fp, zbuf, zs, N, Dz, nl, fN, tw, chained);
         }
         FBS_CUDA(cudaGetLastError());
     }
@@ -1355,7 +1355,7 @@ void launch_count_fields_fp64_impl(Plan &p, double *noct, int bin0, int nb, doub
         auto k = inv_x_kernel<double, true>;
         allow_smem(k, sm);
         dim3 grid(max_inv_x_grid(p, bin0, nb, nl), nb);
-        k<<<grid, kThreads, sm, p.stream>>>(p.d_box, p.boxM, d_geom_grp, 0, A64, nl, p.fM, p.d_tw64, wtab, nullptr);
+        k<<<grid, kThreads, sm, p.stream>>>(p.d_box, p.boxM, d_geom_grp, 0, A64, nl, p.fM, p.d_tw64, wtab, nullptr, 0);
         FBS_CUDA(cudaGetLastError());
     }
     {
@@ -1363,7 +1363,7 @@ void launch_count_fields_fp64_impl(Plan &p, double *noct, int bin0, int nb, doub
         auto k = inv_y_kernel<double>;
         allow_smem(k, sm);
         dim3 grid((max_dzb(p, bin0, nb) + nl - 1) / nl, H, nb);
-        k<<<grid, kThreads, sm, p.stream>>>(A64, d_geom_grp, 0, N, 0, G64, 0, nl, p.fM, p.d_tw64);
+        k<<<grid, kThreads, sm, p.stream>>>(A64, d_geom_grp, 0, N, 0, G64, 0, nl, p.fM, p.d_tw64, 0);
         FBS_CUDA(cudaGetLastError());
     }
     {
@@ -1372,7 +1372,7 @@ void launch_count_fields_fp64_impl(Plan &p, double *noct, int bin0, int nb, doub
         allow_smem(k, sm);
         dim3 grid((H + 2 * nl - 1) / (2 * nl), H, nb);
         k<<<grid, kThreads, sm, p.stream>>>(G64, d_geom_grp, 0, N, 0, noct, (long long)H * H * H,
-                                            nullptr, nl, p.fM, p.d_tw64);
+                                            nullptr, nl, p.fM, p.d_tw64, 0);
         FBS_CUDA(cudaGetLastError());
     }
 }
