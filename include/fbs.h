@@ -392,7 +392,8 @@ fbs_status fbs_trispectrum_diagonal(fbs_plan *plan, const float *field, double *
  * Non-cubic grids and complex fields (Sec. 2: its footnote on non-cubic data,
  * and the remark that Eq. Jeong_gen applies to complex data through complex
  * DFTs).  A separate plan type on the whole grid, FP32 transforms and
- * products with FP64 sums, bispectrum and power spectrum.
+ * products, summed as FP32 pairs (48 bits) per thread and in FP64 across
+ * threads, bispectrum and power spectrum.
  *
  * fbs_gplan_create -- grid n[3] = (N_x, N_y, N_z), each 2^a 3^b in 2..512;
  * box L[3] = (L_x, L_y, L_z) > 0; edges[nbins+1] ascending, physical k.  Mode
