@@ -63,8 +63,8 @@ typedef enum {
 enum {
     FBS_PREC_FP32 = 0,    /* CUDA-core FP32 products, FP64 cross-block sums      */
     FBS_PREC_BF16X3 = 1,  /* tcgen05 tensor cores, BF16 hi/lo split: hi*hi, hi*lo
-                           * and lo*hi (lo*lo too in triplet jobs of the shared-
-                           * operand contraction and of FBS_OPT_TC_STACK)       */
+                           * and lo*hi (lo*lo too in the shared-operand
+                           * contraction and with FBS_OPT_TC_STACK)             */
     FBS_PREC_BF16 = 2     /* tcgen05 tensor cores, plain BF16 (error reported)   */
 };
 
