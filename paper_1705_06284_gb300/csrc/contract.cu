@@ -716,7 +716,7 @@ void launch_contract_fp32(Plan &p, const float *islab, long long npts, long long
     const int G = (num_sms() - one * per) * 33 > num_sms() ? std::max(1, 2 * num_sms() / per) : one;
     dim3 grid(std::min(G, p.part_blocks), job.nblocks, nf);
     const auto run = [&](auto k) {
-        FBS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        allow_smem(k);
         k<<<grid, kCThreads, sm, p.stream>>>(islab, slab_stride, npts, p.nbins, job.d_groups, job.d_rows, job.d_iout,
                                              job.d_blocks, t.nitems,
                                              part_batch ? part_batch : quads ? p.d_qpart : p.d_tpart, p.part_blocks,
@@ -821,7 +821,7 @@ void launch_count_contraction(Plan &p, const double *noct, int nbins_all, int, c
     AsyncBuf pbuf((size_t)blocks * nitems * sizeof(double), p.stream, "count partials");
     double *part = pbuf.as<double>();
     KTimer tm(p, KC_COUNT);
-    FBS_CUDA(cudaFuncSetAttribute(count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    allow_smem(count_kernel);
     dim3 g(blocks, ngrp);
     count_kernel<<<g, 256, sm, p.stream>>>(noct, nbins_all, H, d_items, arity, nitems, grp, part, kCntChunk);
     FBS_CUDA(cudaGetLastError());

@@ -734,7 +734,7 @@ void launch_gram(Plan &p, bool fused, const float *islab, long long npts, long l
     job.last_S = S;
     const auto run = [&](auto kernel, auto units) {
         std::copy(job.units.begin(), job.units.end(), units.u);
-        FBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        allow_smem(kernel);
         kernel<<<dim3(G, job.ngroups, nf), kGThreads, sm, p.stream>>>(
             fmap, npts, p.nbins, job.d_groups, job.d_tables, units, job.d_iout, nitems_total, part, p.part_blocks, F,
             S, lanes, job.maxatoms, p.first_slab, p.root().d_errbuf, p.tc_wait_limit > 0 ? p.tc_wait_limit : kWaitCycles);

@@ -1458,7 +1458,7 @@ static bool launch_wide(Plan &p, const float *islab, long long npts, long long s
     (quads ? p.qrows : p.trows) = G;
     if (p.first_slab) FBS_CUDA(cudaMemsetAsync(part, 0, (size_t)G * t.nitems * sizeof(double), p.stream));
     KTimer tm(p, quads ? KC_QUAD_TC : KC_CONTRACT_TC);
-    FBS_CUDA(cudaFuncSetAttribute(contract_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    allow_smem(contract_wide_kernel);
     dim3 grid(G, ngrp);
     contract_wide_kernel<<<grid, kWideThreads, sm, p.stream>>>(
         islab, slab_stride, npts, p.nbins, w.nleft, w.d_left, w.d_rights, w.nright, w.d_item_out, t.nitems,
@@ -1582,8 +1582,7 @@ static void launch_job(Plan &p, TcJob &job, const float *islab, long long npts, 
 #define FBS_TC_LAUNCH(A, S, W, K, F)                                                                  \
     if (nst == A && nstg == S && aw == W && ka == K && (ifeed != nullptr) == F) {                   \
         launched = true;                                                                              \
-        FBS_CUDA(cudaFuncSetAttribute(contract_tc_kernel<A, S, W, K, F>,                                 \
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));          \
+        allow_smem(contract_tc_kernel<A, S, W, K, F>);                                                \
         contract_tc_kernel<A, S, W, K, F><<<grid, kTcThreads, sm, p.stream>>>(                          \
             fmap, npts, p.nbins, job.Npad, tstr, job.ninner, job.d_inner, job.d_pairs, job.npairs,      \
             job.d_grp, job.d_iout, nitems_total, part, x3, flush_every, st.d_err, tc_wait_limit(p),     \

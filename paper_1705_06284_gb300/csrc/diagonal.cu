@@ -116,7 +116,7 @@ void launch_diag_gram(Plan &p, const float2 *FA, int na, const float2 *FB, int n
     if (ntasks > 0) {
         const int per_block = kDiagThreads * (nq > kDiagThreads ? 2 : 1);
         const auto kernel = nq > kDiagThreads ? diag_gram_kernel<2> : diag_gram_kernel<1>;
-        FBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        allow_smem(kernel);
         dim3 grid(ntasks, (nq + per_block - 1) / per_block);
         kernel<<<grid, kDiagThreads, sm, p.stream>>>(FA, na, FB, rows, per, d_uv, nq, d_idx, d_tasks, chunk,
                                                                part);

@@ -21,6 +21,12 @@ struct Failure {
 // Throws Failure on CUDA error (caught at the ABI boundary).
 void check_cuda(cudaError_t e, const char *what);
 #define FBS_CUDA(call) ::fbs::check_cuda((call), #call)
+// Allow `kernel` all the dynamic shared memory that the device has beside its
+// static arrays.  The limit is the process's, not the launch's: set to each
+// launch's own size, one thread lowers it between another's set and launch,
+// which is then refused.
+void allow_smem(const void *kernel);
+template <class K> void allow_smem(K *kernel) { allow_smem(reinterpret_cast<const void *>(kernel)); }
 
 // ---------------------------------------------------------------- FFT plan
 // Radix factorisation of a length-n transform (n = 2^a 3^b <= 512).

@@ -45,9 +45,8 @@ static int lines_per_cta(int N) {
 }
 
 template <typename K>
-static void allow_smem(K kernel, size_t bytes) {
-    if (bytes > 48 * 1024)
-        FBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+static void allow_smem(K *kernel, size_t bytes) {
+    if (bytes > 48 * 1024) allow_smem(kernel);
 }
 
 // CTAs of a kernel that fit on the device at once (dynamic shared memory
@@ -57,7 +56,7 @@ static int resident_ctas(K kernel, int threads, size_t dyn) {
     int dev = 0, sms = 0, per = 0;
     FBS_CUDA(cudaGetDevice(&dev));
     FBS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    FBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    allow_smem(kernel);
     FBS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, dyn));
     return sms * std::max(1, per);
 }

@@ -374,7 +374,7 @@ void transform3(fbs_gplan &g, typename V2<T>::t *d, typename V2<T>::t *const *tw
         const int nl = std::max(1, std::min(16, (int)((64 * 1024) / (2 * n * sizeof(typename V2<T>::t)))));
         const size_t sm = 2 * (size_t)nl * n * sizeof(typename V2<T>::t);
         auto k = axis_fft_kernel<T, DIR>;
-        if (sm > 48 * 1024) FBS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        if (sm > 48 * 1024) allow_smem(k);
         const long long nlines = g.npix / n;
         k<<<(unsigned)((nlines + nl - 1) / nl), kT, sm, g.stream>>>(d, g.n[0], g.n[1], g.n[2], axis, g.f[axis],
                                                                    tw[axis], nl);
@@ -390,7 +390,7 @@ void gfft_pass(fbs_gplan &g, const float2 *src, float2 *dst, int axis, int nb) {
     const int nl = std::max(1, std::min(16, (int)((64 * 1024) / (2 * (n + 1) * sizeof(float2)))));
     const size_t sm = 2 * (size_t)nl * (n + 1) * sizeof(float2);
     auto k = gfft_kernel<DIR>;
-    if (sm > 48 * 1024) FBS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (sm > 48 * 1024) allow_smem(k);
     const long long nlines = g.npix / n;
     k<<<dim3((unsigned)((nlines + nl - 1) / nl), nb), kT, sm, g.stream>>>(src, dst, g.n[0], g.n[1], g.n[2], axis,
                                                                          g.f[axis], g.d_tw[axis], nl, g.d_bin, g.d_R);
@@ -541,8 +541,7 @@ void gplan_run(fbs_gplan &g, const float *field) {
     while (slices < kT / 32 && 2 * slices * nitems <= kT) slices *= 2;
     const int per = kT / slices;
     const int tile = (int)std::max<long long>(1, std::min<long long>(256, 32 * 1024 / (nb * 8)));
-    const size_t sm = (size_t)tile * nb * sizeof(float2);
-    FBS_CUDA(cudaFuncSetAttribute(ctriple_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    const size_t sm = (size_t)tile * nb * sizeof(float2);  // at most 32 KB
     const int ny = (nitems + per - 1) / per;
     for (int y0 = 0; y0 < ny; y0 += 65535) {
         const int c0 = y0 * per;

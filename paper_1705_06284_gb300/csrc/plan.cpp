@@ -23,6 +23,7 @@
 #include <chrono>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -73,6 +74,26 @@ void budget_reserve(long long bytes) {
 }
 
 void budget_release(long long bytes) { g_in_use.fetch_sub(bytes); }
+
+void allow_smem(const void *kernel) {
+    static std::mutex mtx;
+    static std::map<std::pair<const void *, int>, int> limits;  // by kernel and device
+    int dev = 0, limit = 0;
+    FBS_CUDA(cudaGetDevice(&dev));
+    {
+        std::lock_guard<std::mutex> lock(mtx);
+        auto it = limits.find({kernel, dev});
+        if (it == limits.end()) {
+            cudaFuncAttributes a{};
+            int most = 0;
+            FBS_CUDA(cudaFuncGetAttributes(&a, kernel));
+            FBS_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+            it = limits.emplace(std::make_pair(kernel, dev), most - (int)a.sharedSizeBytes).first;
+        }
+        limit = it->second;
+    }
+    FBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
+}
 
 AsyncBuf::AsyncBuf(size_t n, cudaStream_t s, const char *what) : stream(s) {
     if (n == 0) n = 16;

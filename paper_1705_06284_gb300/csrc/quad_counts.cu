@@ -284,8 +284,7 @@ void exact_quad_counts(Plan &p, const double *noct, const std::vector<int> &item
     FBS_CUDA(cudaMemsetAsync(dist.ptr, 0, sizeof(unsigned long long), p.stream));
     const int nl = std::max(1, std::min(16, (96 * 1024) / (2 * M * (int)sizeof(double2))));
     const size_t esm = 2 * (size_t)nl * M * sizeof(double2);
-    if (esm > 48 * 1024)
-        FBS_CUDA(cudaFuncSetAttribute(even_dft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm));
+    if (esm > 48 * 1024) allow_smem(even_dft_kernel);
     const long long HH = (long long)H * H;
     const int eblocks = (int)(((HH + 1) / 2 + nl - 1) / nl);
     const int sblocks = (int)std::min<long long>(4096, (H3 + kThr - 1) / kThr);
