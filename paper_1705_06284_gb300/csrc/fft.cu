@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(T *LP) inv_y_reg_kernel(const float2 *__restri
     const float2 *in = A + g.A_off + (long long)x * g.Db * g.Dzb;
     const bool full = g.Db == N;  // the bin's box spans the whole axis
     const int Rb = full ? N / 2 : (g.Db - 1) / 2;
-    const int mz2 = mz * mz, hi2 = (int)g.thr_hi;          // (at most 3 N^2 / 4)
+    const int mz2 = mz * mz, hi2 = (int)g.thr_hi;  // at most 3 N^2 / 4 + 1 of the input grid
 #pragma unroll 1
     for (int j = 0; j < N1 / T; ++j) {
         const int n1 = t + T * j;
@@ -919,7 +919,7 @@ __global__ void __launch_bounds__(T *LP) inv_x_reg_kernel(const float2 *__restri
     const int l = threadIdx.x % LP, t = threadIdx.x / LP;
     const int mz = jz0 + l;
     const bool col = mz < g.Dzb;
-    const int r2 = my * my + mz * mz, lo2 = (int)g.thr_lo, hi2 = (int)g.thr_hi;  // at most 3 N^2 / 4 < 2^31
+    const int r2 = my * my + mz * mz, lo2 = (int)g.thr_lo, hi2 = (int)g.thr_hi;  // at most 3 N^2 / 4 + 1
     const float2 *in = box + g.box_off + (long long)box_index(my, bg.D) * bg.Dz + (col ? mz : 0);
     const long long xs = (long long)bg.D * bg.Dz;  // box stride along x
     const bool fullx = bg.D == N;

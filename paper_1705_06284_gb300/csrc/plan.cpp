@@ -269,12 +269,15 @@ static void build_level_geometry(Plan &root, Plan &lv) {
     const int M = lv.M;
     lv.nbins = (int)lv.gbin.size();
     lv.geom.assign(lv.nbins, BinGeom{});
+    // thresholds past the grid's largest |m|^2 are the same shell (aliased
+    // plans take any top edge; the kernels compare in 32 bits)
+    const long long past = 3LL * (root.N / 2) * (root.N / 2) + 1;
     long long aoff = 0;
     for (int b = 0; b < lv.nbins; ++b) {
         const int gb = lv.gbin[b];
         BinGeom &g = lv.geom[b];
-        g.thr_lo = root.thr[gb];
-        g.thr_hi = root.thr[gb + 1];
+        g.thr_lo = std::min(root.thr[gb], past);
+        g.thr_hi = std::min(root.thr[gb + 1], past);
         g.empty = 0;  // levels hold non-empty bins only
         g.Rb = std::min(isqrt_floor(g.thr_hi - 1), M / 2);
         g.Db = (2 * g.Rb + 1 > M) ? M : 2 * g.Rb + 1;
