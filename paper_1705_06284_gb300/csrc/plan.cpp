@@ -1348,27 +1348,36 @@ static void run_diagonal(Plan &p, const float *field) {
         lv.d_G = G0;
         lv.slab = slab0;
         const long long per = (long long)dl.bx.D * dl.bx.D * dl.bx.Dz;  // complex elements of one pair spectrum
-        // pair spectra in groups of 4 GiB at most, few enough to stage one mode of two groups
-        const int K = (int)std::max<long long>(1, std::min<long long>({np, 6000, (4LL << 30) / (per * 8)}));
+        // pair spectra in groups of 4 GiB at most, few enough to stage one mode of
+        // two groups (FBS_DIAG_GROUP: fewer pairs to a group)
+        long long most = 6000;
+        if (const char *e = getenv("FBS_DIAG_GROUP")) most = std::min(most, std::max(1LL, atoll(e)));
+        const int K = (int)std::max<long long>(1, std::min<long long>({np, most, (4LL << 30) / (per * 8)}));
         const int ng = (np + K - 1) / K;
-        // forward transforms of as many products at once as a gigabyte of scratch holds
-        const long long fwd = (long long)M * M * dl.bx.Dz + (long long)M * dl.bx.D * dl.bx.Dz;
-        int F = (int)std::max<long long>(1, std::min<long long>(std::min(np, K), (1LL << 30) / (fwd * 8)));
-        const auto scratch = [&] {
-            return std::unique_ptr<AsyncBuf>(new AsyncBuf((size_t)F * fwd * sizeof(float2), p.stream, "diagonal scratch"));
-        };
-        std::unique_ptr<AsyncBuf> zy;
-        try {
-            zy = scratch();
-        } catch (const Failure &) {  // (no room for that: one at a time)
-            F = 1;
-            zy = scratch();
-        }
-        float2 *const zb = zy->as<float2>(), *const yb = zb + (long long)F * M * M * dl.bx.Dz;
         AsyncBuf FA((size_t)std::min(np, K) * per * sizeof(float2), p.stream, "pair spectra");
         AsyncBuf FB(ng > 1 ? (size_t)K * per * sizeof(float2) : 16, p.stream, "pair spectra");
+        // forward transforms of as many products at once as a gigabyte of scratch
+        // holds, partial sums of as many quadruplets as 64 MiB; where that is
+        // refused, one product and the partials that the memory of one more
+        // field holds
         const int nql = (int)lv.nquad.size();
-        AsyncBuf part((size_t)std::max(1, dl.ntasks) * nql * sizeof(double), p.stream, "diagonal scratch");
+        const long long fwd = (long long)M * M * dl.bx.Dz + (long long)M * dl.bx.D * dl.bx.Dz;
+        const long long per_quad = 8LL * std::max(1, dl.ntasks);
+        int F = 1, Q = 1;
+        std::unique_ptr<AsyncBuf> zy, part;
+        for (const bool least : {false, true}) {
+            F = least ? 1 : (int)std::max<long long>(1, std::min<long long>(std::min(np, K), (1LL << 30) / (fwd * 8)));
+            Q = (int)std::max<long long>(1, std::min<long long>(nql, (least ? 4 * M3 : 64LL << 20) / per_quad));
+            try {
+                zy.reset(new AsyncBuf((size_t)F * fwd * sizeof(float2), p.stream, "diagonal scratch"));
+                part.reset(new AsyncBuf((size_t)Q * per_quad, p.stream, "diagonal scratch"));
+                break;
+            } catch (const Failure &) {
+                zy.reset();
+                if (least) throw;
+            }
+        }
+        float2 *const zb = zy->as<float2>(), *const yb = zb + (long long)F * M * M * dl.bx.Dz;
         auto compute = [&](int g, float2 *dst) {
             const int end = std::min(np, (g + 1) * K);
             for (int j = g * K; j < end; j += F) {
@@ -1378,10 +1387,15 @@ static void run_diagonal(Plan &p, const float *field) {
             }
         };
         const double scale = 1.0 / ((double)M3 * (double)M3);  // DFT_M of a pair product is M^3 F_ab
+        auto gram = [&](int na, int nbr, const int2 *d_uv, const int *d_qout, int nq) {
+            for (int q0 = 0; q0 < nq; q0 += Q)
+                launch_diag_gram(lv, FA.as<float2>(), na, FB.as<float2>(), nbr, per, d_uv + q0, std::min(Q, nq - q0),
+                                 dl.d_idx, dl.d_tasks, dl.ntasks, dl.d_tstart, nd, d_qout + q0, scale,
+                                 part->as<double>(), ds.d_num);
+        };
         if (ng == 1) {
             compute(0, FA.as<float2>());
-            launch_diag_gram(lv, FA.as<float2>(), np, nullptr, 0, per, dl.d_uv, nql, dl.d_idx, dl.d_tasks, dl.ntasks,
-                             dl.d_tstart, nd, dl.d_qout, scale, part.as<double>(), ds.d_num);
+            gram(np, 0, dl.d_uv, dl.d_qout, nql);
             continue;
         }
         for (int gi = 0; gi < ng; ++gi) {
@@ -1406,9 +1420,7 @@ static void run_diagonal(Plan &p, const float *field) {
                                          p.stream));
                 FBS_CUDA(cudaMemcpyAsync(d_q.ptr, qout.data(), qout.size() * sizeof(int), cudaMemcpyHostToDevice,
                                          p.stream));
-                launch_diag_gram(lv, FA.as<float2>(), na, FB.as<float2>(), nbr, per, d_uv.as<int2>(), (int)uv.size(),
-                                 dl.d_idx, dl.d_tasks, dl.ntasks, dl.d_tstart, nd, d_q.as<int>(), scale,
-                                 part.as<double>(), ds.d_num);
+                gram(na, nbr, d_uv.as<int2>(), d_q.as<int>(), (int)uv.size());
                 FBS_CUDA(cudaStreamSynchronize(p.stream));  // uv and qout go out of scope
             }
         }
