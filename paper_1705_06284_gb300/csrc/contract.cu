@@ -675,23 +675,19 @@ static void build_fp32_job(Plan &p, const TaskList &t, bool quads, FpJob &job) {
         groups.push_back(g);
     }
     close();
-    const auto up = [&](const void *v, size_t bytes) {
-        void *d = p.dalloc(std::max<size_t>(bytes, 16));
-        FBS_CUDA(cudaMemcpyAsync(d, v, bytes, cudaMemcpyHostToDevice, p.stream));
-        return d;
-    };
-    job.d_groups = (FpGroup *)up(groups.data(), groups.size() * sizeof(FpGroup));
-    job.d_rows = (FpRow *)up(rows.data(), rows.size() * sizeof(FpRow));
-    job.d_iout = (int *)up(iout.data(), iout.size() * sizeof(int));
-    job.d_blocks = (int4 *)up(blocks.data(), blocks.size() * sizeof(int4));
-    FBS_CUDA(cudaStreamSynchronize(p.stream));  // host tables go out of scope
+    TableUpload up(p);
+    job.d_groups = up.put(groups);
+    job.d_rows = up.put(rows);
+    job.d_iout = up.put(iout);
+    job.d_blocks = up.put(blocks);
+    up.wait();
     job.nblocks = (int)blocks.size();
     job.built = true;
 }
 
 // Tables of a level's FP32 contraction, built when the plan first has a use for
-// them (its creation or a change of precision, never inside an evaluation that
-// a caller may be capturing).
+// them: its creation, or the first FP32 evaluation of one made for another
+// precision.
 void prepare_fp32(Plan &p, bool trip, bool quads) {
     if (trip && !p.fpt.built && p.ttask.nitems > 0) build_fp32_job(p, p.ttask, false, p.fpt);
     if (quads && !p.fpq.built && p.qtask.nitems > 0) build_fp32_job(p, p.qtask, true, p.fpq);

@@ -515,13 +515,6 @@ static size_t gram_smem(const Plan &p, const GramJob &j, int F, int S) {
 constexpr size_t kGramSmemCap = 225 * 1024;
 constexpr int kMaxUnits = 80;  // of all groups: 11.5 KB of kernel arguments
 
-template <typename T>
-static T *gram_upload(Plan &p, const std::vector<T> &v) {
-    T *d = (T *)p.dalloc(std::max<size_t>(1, v.size()) * sizeof(T));
-    FBS_CUDA(cudaMemcpyAsync(d, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, p.stream));
-    return d;
-}
-
 // Eight rows' factor offsets so that rows 0..3 have one x and rows 4..7
 // another, by swapping the factors of single rows (empty rows take any): true
 // when that is possible.
@@ -633,10 +626,11 @@ static void finish_gram(Plan &p, GramJob &job, const std::vector<GramRows> &grou
     }
     job.ngroups = (int)hg.size();
     if ((int)job.units.size() > kMaxUnits || gram_smem(p, job, 2, 2) > kGramSmemCap) return;
-    job.d_groups = gram_upload(p, hg);
-    job.d_tables = gram_upload(p, ht);
-    job.d_iout = gram_upload(p, iout);
-    FBS_CUDA(cudaStreamSynchronize(p.stream));  // host tables go out of scope
+    TableUpload up(p);
+    job.d_groups = up.put(hg);
+    job.d_tables = up.put(ht);
+    job.d_iout = up.put(iout);
+    up.wait();
     job.usable = true;
 }
 

@@ -1094,19 +1094,12 @@ static void finish_job(Plan &p, TcJob &job, const std::vector<TcPair> &hp, const
     if (p.nbins > 256) return;  // one TMA box spans every bin
     if (tc_smem_bytes(p.nbins, job.Npad, job.maxloc, job.maxtiles, 2) > smem_cap) return;
     if ((((job.maxtiles * tile_stride(job.Npad)) + 31) / 32) * 32 + 2 * kAStageCols > 512) return;
-    job.d_pairs = (TcPair *)p.dalloc(hp.size() * sizeof(TcPair));
-    FBS_CUDA(cudaMemcpyAsync(job.d_pairs, hp.data(), hp.size() * sizeof(TcPair), cudaMemcpyHostToDevice,
-                             p.stream));
-    job.d_inner = (int2 *)p.dalloc(inner.size() * sizeof(int2));
-    FBS_CUDA(cudaMemcpyAsync(job.d_inner, inner.data(), inner.size() * sizeof(int2), cudaMemcpyHostToDevice,
-                             p.stream));
-    job.d_iout = (int *)p.dalloc(std::max<size_t>(1, iout.size()) * sizeof(int));
-    FBS_CUDA(cudaMemcpyAsync(job.d_iout, iout.data(), iout.size() * sizeof(int), cudaMemcpyHostToDevice,
-                             p.stream));
-    job.d_grp = (int *)p.dalloc(job.grp.size() * sizeof(int));
-    FBS_CUDA(cudaMemcpyAsync(job.d_grp, job.grp.data(), job.grp.size() * sizeof(int),
-                             cudaMemcpyHostToDevice, p.stream));
-    FBS_CUDA(cudaStreamSynchronize(p.stream));  // host tables go out of scope
+    TableUpload up(p);
+    job.d_pairs = up.put(hp);
+    job.d_inner = up.put(inner);
+    job.d_iout = up.put(iout);
+    job.d_grp = up.put(job.grp);
+    up.wait();
     job.usable = true;
 }
 
@@ -1227,10 +1220,9 @@ static void attach_feed(Plan &p, TcJob &job, const std::vector<TcPair> &hp, cons
         feed[it->second] = n;
     }
     job.nsingle = nbuild;
-    job.d_ifeed = (int *)p.dalloc(feed.size() * sizeof(int));
-    FBS_CUDA(cudaMemcpyAsync(job.d_ifeed, feed.data(), feed.size() * sizeof(int), cudaMemcpyHostToDevice,
-                             p.stream));
-    FBS_CUDA(cudaStreamSynchronize(p.stream));
+    TableUpload up(p);
+    job.d_ifeed = up.put(feed);
+    up.wait();
 }
 
 // FP64 partial rows of a fused pass (once per level).
@@ -1421,12 +1413,11 @@ static void build_wide(Plan &p, bool quads, WideJob &w) {
         const int n = R[r1].first + __builtin_popcountll(R[r1].mask) - R[r0].first;
         w.maxloc = std::max(w.maxloc, n);
     }
-    w.d_left = (int2 *)p.dalloc(left.size() * sizeof(int2));
-    FBS_CUDA(cudaMemcpyAsync(w.d_left, left.data(), left.size() * sizeof(int2), cudaMemcpyHostToDevice, p.stream));
-    w.d_rights = (WideRight *)p.dalloc(R.size() * sizeof(WideRight));
-    FBS_CUDA(cudaMemcpyAsync(w.d_rights, R.data(), R.size() * sizeof(WideRight), cudaMemcpyHostToDevice, p.stream));
-    w.d_item_out = (int *)p.dalloc(out.size() * sizeof(int));
-    FBS_CUDA(cudaMemcpyAsync(w.d_item_out, out.data(), out.size() * sizeof(int), cudaMemcpyHostToDevice, p.stream));
+    TableUpload up(p);
+    w.d_left = up.put(left);
+    w.d_rights = up.put(R);
+    w.d_item_out = up.put(out);
+    up.wait();
     w.usable = true;
 }
 

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -278,7 +279,7 @@ struct Plan {
     cudaEvent_t ev_err = nullptr;
     bool err_recorded = false;
     float *d_field = nullptr;    // staging for host fields
-    cudaStream_t copy_stream = nullptr;   // host-field copies (overlap work queued on `stream`)
+    cudaStream_t copy_stream = nullptr;   // host fields and tables (overlap work queued on `stream`)
     cudaEvent_t ev_field_ready = nullptr; // staged copy landed (the plan's stream waits on it)
     cudaEvent_t ev_field_free = nullptr;  // the forward transform is done with the staging buffer
     bool field_free_recorded = false;
@@ -329,6 +330,33 @@ struct Plan {
     void tic(int cls, int &slot);
     void toc(int slot);
     void flush_times();
+};
+
+// Allows allocations on this thread whatever stream is being captured.
+struct OffCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    OffCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~OffCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// Host tables to device memory of the plan, on its copy stream: tables that an
+// evaluation finds missing are there when its kernels run, also when the plan's
+// stream is being captured (nothing here becomes part of it).
+class TableUpload {
+  public:
+    explicit TableUpload(Plan &plan) : p(plan), stream(plan.root().copy_stream) {}
+    TableUpload(const TableUpload &) = delete;
+    template <typename T> T *put(const std::vector<T> &v) {
+        T *d = (T *)p.dalloc(std::max<size_t>(1, v.size()) * sizeof(T));
+        FBS_CUDA(cudaMemcpyAsync(d, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, stream));
+        return d;
+    }
+    void wait() { FBS_CUDA(cudaStreamSynchronize(stream)); }  // before the host tables go out of scope
+
+  private:
+    OffCapture off;
+    Plan &p;
+    cudaStream_t stream;
 };
 
 // Bracket a launch with timing events when FBS_FLAG_TIMING is set.

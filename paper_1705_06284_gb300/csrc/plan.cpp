@@ -120,6 +120,7 @@ void *Plan::dalloc(size_t bytes) {
     void *ptr = nullptr;
     if (bytes == 0) bytes = 16;
     budget_reserve((long long)bytes);
+    OffCapture off;
     cudaError_t e = cudaMalloc(&ptr, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -678,6 +679,7 @@ static void create_plan(Plan &p, const double *edges, const void *blob = nullptr
     p.box.Dz = std::min(Rmax, N / 2) + 1;
     p.M = N;
 
+    FBS_CUDA(cudaStreamCreateWithFlags(&p.copy_stream, cudaStreamNonBlocking));
     // forward twiddles, spectrum box, timeout flags
     upload_forward_twiddles(p);
     p.d_box = (float2 *)p.dalloc((size_t)p.box.D * p.box.D * p.box.Dz * sizeof(float2));
@@ -896,7 +898,6 @@ static void create_plan(Plan &p, const double *edges, const void *blob = nullptr
 
     // per-field buffers of the root
     p.d_field = (float *)p.dalloc((size_t)N * N * N * sizeof(float));
-    FBS_CUDA(cudaStreamCreateWithFlags(&p.copy_stream, cudaStreamNonBlocking));
     FBS_CUDA(cudaEventCreateWithFlags(&p.ev_field_ready, cudaEventDisableTiming));
     FBS_CUDA(cudaEventCreateWithFlags(&p.ev_field_free, cudaEventDisableTiming));
     FBS_CUDA(cudaEventCreateWithFlags(&p.ev_err, cudaEventDisableTiming));
@@ -1676,13 +1677,9 @@ fbs_status fbs_plan_set_precision(fbs_plan *plan, int precision) {
         set_error("bad plan or precision");
         return FBS_ERR_ARG;
     }
-    FBS_GUARD_BEGIN
-    if (precision == FBS_PREC_FP32)
-        for (Plan *lv : plan->levels) prepare_fp32(*lv, true, false);
     plan->precision = precision;
     for (Plan *lv : plan->levels) lv->precision = precision;
     return FBS_OK;
-    FBS_GUARD_END
 }
 
 static bool set_plan_option(Plan *plan, int option, int value);
