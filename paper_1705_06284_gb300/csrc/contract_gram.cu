@@ -218,7 +218,7 @@ __device__ __forceinline__ void form_unit(const unsigned char *st, const GramUni
 
 // grid: (point-range CTAs, groups, fields of a batch).
 // F field stages and S operand stages in shared memory.
-template <int CAP, bool FIXED>
+template <int CAP>
 __global__ void __launch_bounds__(kGThreads, 1)
     contract_gram_kernel(const __grid_constant__ CUtensorMap fmap, long long npts, int nbins,
                          const GramGroup *__restrict__ groups, const GramTable *__restrict__ tables,
@@ -291,11 +291,9 @@ __global__ void __launch_bounds__(kGThreads, 1)
 
     if (warp < kProd) {
         // ================= producers =================
-        // FIXED: a warp forms one unit of every `lanes`-th step; lanes divides F
-        // and S, so a slot's previous use was this warp's own and the parity it
-        // waits for is never two phases ahead.  Otherwise (more units than
-        // warps) the units of a step go round all warps, each of which has one
-        // or more in every step.
+        // A warp forms one unit of every `lanes`-th step; lanes divides F and S, so
+        // a slot's previous use was this warp's own and the parity it waits for is
+        // never two phases ahead.
         const uint32_t lane_off = (uint32_t)((lane >> 3) * 1024 + (lane & 7) * 128);
         const unsigned char *const fl = f0 + 8 * lane;
         unsigned char *const xl = X0 + lane_off;
@@ -313,31 +311,16 @@ __global__ void __launch_bounds__(kGThreads, 1)
                 mbar_arrive(&bars.fempty[fs]);
             }
         };
-        if (FIXED) {
-            if (warp < lanes * nu) {
-                const GramUnit U = units.u[g.unit0 + warp % nu];
-                int step = warp / nu, fs = step, xs = step;
-                uint32_t fph = 0, xph = 0;
-                for (; step < nsteps; step += lanes) {
-                    wait_step(step, fs, fph, xs, xph);
-                    form_unit(fl + fs * fstage, U, xl + xs * xstage, lane);
-                    hand_over(fs, xs);
-                    if ((fs += lanes) >= F) { fs -= F; fph ^= 1u; }
-                    if ((xs += lanes) >= S) { xs -= S; xph ^= 1u; }
-                }
-            }
-        } else {
-            int u = warp, fs = 0, xs = 0;
+        if (warp < lanes * nu) {
+            const GramUnit U = units.u[g.unit0 + warp % nu];
+            int step = warp / nu, fs = step, xs = step;
             uint32_t fph = 0, xph = 0;
-            for (int step = 0; step < nsteps; ++step) {
+            for (; step < nsteps; step += lanes) {
                 wait_step(step, fs, fph, xs, xph);
-                for (; u < nu; u += kProd) {
-                    form_unit(fl + fs * fstage, units.u[g.unit0 + u], xl + xs * xstage, lane);
-                    hand_over(fs, xs);
-                }
-                u -= nu;
-                if (++fs == F) { fs = 0; fph ^= 1u; }
-                if (++xs == S) { xs = 0; xph ^= 1u; }
+                form_unit(fl + fs * fstage, U, xl + xs * xstage, lane);
+                hand_over(fs, xs);
+                if ((fs += lanes) >= F) { fs -= F; fph ^= 1u; }
+                if ((xs += lanes) >= S) { xs -= S; xph ^= 1u; }
             }
         }
     } else if (warp < kMma) {
@@ -625,7 +608,9 @@ static void finish_gram(Plan &p, GramJob &job, const std::vector<GramRows> &grou
         job.nbrows = std::max(job.nbrows, 8 * g.nbch);
     }
     job.ngroups = (int)hg.size();
-    if ((int)job.units.size() > kMaxUnits || gram_smem(p, job, 2, 2) > kGramSmemCap) return;
+    // (a group's units never outnumber the producer warps that form them: at most
+    // 64 rows of A and 256 of B in units of 16)
+    if (job.maxunits > kProd || (int)job.units.size() > kMaxUnits || gram_smem(p, job, 2, 2) > kGramSmemCap) return;
     TableUpload up(p);
     job.d_groups = up.put(hg);
     job.d_tables = up.put(ht);
@@ -679,7 +664,9 @@ static void build_gram_fused(Plan &p, GramJob &job) {
 // of the tensor-memory kernel).  Faster than that kernel at every job it can
 // hold (the figures above; 64^3, 12 bins, 30 -> 19 us; 192^3, 48 bins, 787 ->
 // 746 us), so there is no further rule on sizes: what does not fit (more than
-// 64 bins on operand A, more than 256 rows or kMaxUnits units) stays there.
+// 64 bins on operand A, more than 256 rows or kMaxUnits units, or two operand
+// and two field stages past kGramSmemCap: 46 to 48 linear bins at 256^3 and
+// above) stays there.
 static bool gram_options(const Plan &p) {
     return !p.gram_off && p.precision == FBS_PREC_BF16X3 && !p.tc_wide && !p.tc_roles && !p.tc_chunk && !p.tc_pairs && !p.tc_merge &&
            !p.tc_bstages && !p.tc_bfroma && !p.tc_stack;
@@ -734,11 +721,9 @@ void launch_gram(Plan &p, bool fused, const float *islab, long long npts, long l
             S, lanes, job.maxatoms, p.first_slab, p.root().d_errbuf, p.tc_wait_limit > 0 ? p.tc_wait_limit : kWaitCycles);
     };
     // the argument block sized for the job (1.7, 3.5 or 11.5 KB)
-    const bool fixed = job.maxunits <= kProd;
-    if (job.units.size() <= 12) run(contract_gram_kernel<12, true>, GramUnits<12>{});
-    else if (job.units.size() <= 24) run(contract_gram_kernel<24, true>, GramUnits<24>{});
-    else if (fixed) run(contract_gram_kernel<kMaxUnits, true>, GramUnits<kMaxUnits>{});
-    else run(contract_gram_kernel<kMaxUnits, false>, GramUnits<kMaxUnits>{});
+    if (job.units.size() <= 12) run(contract_gram_kernel<12>, GramUnits<12>{});
+    else if (job.units.size() <= 24) run(contract_gram_kernel<24>, GramUnits<24>{});
+    else run(contract_gram_kernel<kMaxUnits>, GramUnits<kMaxUnits>{});
     FBS_CUDA(cudaGetLastError());
 }
 
