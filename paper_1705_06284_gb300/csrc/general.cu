@@ -519,12 +519,16 @@ void gplan_build(fbs_gplan &g, const double *edges) {
 
 void gplan_run(fbs_gplan &g, const float *field) {
     const size_t bytes = (size_t)g.npix * sizeof(float2);
+    // read in place where the kernels can: this device's memory or managed memory
     cudaPointerAttributes a;
     bool dev = false;
-    if (cudaPointerGetAttributes(&a, field) == cudaSuccess)
-        dev = a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
-    else
+    if (cudaPointerGetAttributes(&a, field) == cudaSuccess) {
+        int here = 0;
+        FBS_CUDA(cudaGetDevice(&here));
+        dev = (a.type == cudaMemoryTypeDevice && a.device == here) || a.type == cudaMemoryTypeManaged;
+    } else {
         cudaGetLastError();
+    }
     const float2 *in = reinterpret_cast<const float2 *>(field);
     if (!dev || (reinterpret_cast<uintptr_t>(field) & 7)) {
         FBS_CUDA(cudaMemcpyAsync(g.d_in, field, bytes, cudaMemcpyDefault, g.stream));
