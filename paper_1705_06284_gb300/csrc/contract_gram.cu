@@ -727,9 +727,10 @@ void launch_gram(Plan &p, bool fused, const float *islab, long long npts, long l
     FBS_CUDA(cudaGetLastError());
 }
 
-// Job shape diagnostics (fbs_plan_tc_info): false when the job was not launched here.
+// Job shape diagnostics (fbs_plan_tc_info): false when the job was not launched
+// here, or is not with the plan's present options.  Builds nothing.
 bool gram_job_info(Plan &p, bool fused, int32_t *out) {
-    if (!p.gram) return false;
+    if (!p.gram || !gram_options(p)) return false;
     const GramJob &j = fused ? gram_state(p).fused : gram_state(p).trip;
     if (!j.usable || !j.last_S) return false;
     out[0] = out[1] = 1;

@@ -1463,7 +1463,7 @@ static bool launch_wide(Plan &p, const float *islab, long long npts, long long s
 // and of its latest launch the merged flag and points per step / 64.
 void tc_job_info(Plan &p, int which, int32_t *out) {
     for (int i = 0; i < 11; ++i) out[i] = 0;
-    if (which != 1 && p.gram && gram_usable(p, which == 2) && gram_job_info(p, which == 2, out)) return;
+    if (which != 1 && gram_job_info(p, which == 2, out)) return;
     if (!p.tc) return;
     TcState &st = *reinterpret_cast<TcState *>(p.tc);
     const TcJob &j = which == 0 ? st.trip : which == 1 ? st.quad : st.fused;
