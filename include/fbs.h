@@ -314,8 +314,10 @@ fbs_status fbs_trispectrum(fbs_plan *plan, const float *field, double *T, double
  * 3 S2^2 - 3 S4 + the self-conjugate modes' D^4, S2/S4 the shell's sums of
  * |D|^2 and |D|^4) and N_conn the unpaired count (fbs_plan_quads_connected).
  * A Gaussian field's Tc has zero mean.  Tc is NaN where a quadruplet has no
- * unpaired quadruple.  Tc[nquad], T[nquad], B[ntrip], P[nbins]: device or
- * host or NULL; same stream semantics as fbs_bispectrum.
+ * unpaired quadruple.  B and T agree with fbs_trispectrum's within the
+ * precision's rounding (BF16x3 runs on another kernel here).  Tc[nquad],
+ * T[nquad], B[ntrip], P[nbins]: device or host or NULL; same stream semantics
+ * as fbs_bispectrum.
  */
 fbs_status fbs_trispectrum_connected(fbs_plan *plan, const float *field, double *Tc, double *T, double *B,
                                      double *P);

@@ -7,9 +7,10 @@
 // with its writes visible.  Since every block waits before it does anything
 // else, completion is transitive along the chain and buffers may be reused as
 // in an ordinary stream.  `chained` is the kernel's last argument, whether it
-// was launched this way: in an ordinary launch the wait returns at once, but
-// the x stage's tens of thousands of blocks that find nothing to do paid for it
-// (0.47 -> 0.57 ms at 512^3).
+// belongs to such a chain (the forward z pass, which begins one, is launched the
+// ordinary way and only allows the next launch: its wait returns at once).
+// Other launches skip both: the x stage's tens of thousands of blocks that find
+// nothing to do paid for the wait (0.47 -> 0.57 ms at 512^3).
 #pragma once
 
 #include <cuda_runtime.h>

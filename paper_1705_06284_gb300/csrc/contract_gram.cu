@@ -29,10 +29,13 @@
 // compensated FP32 sums per item while the MMAs of the next 1,024 points go to
 // the other half of tensor memory (one tile of B; two tiles take turns).
 //
-// What bounds it: shared memory.  The trispectrum pass of 16 log bins at 256^3
-// takes 1,386 cycles per 64-point step, of which the producers' and the
-// accumulator warps' wavefronts fill 72% and the MMAs' operand reads (128 + N
-// rows of 32 bytes per 16 points) 27%; the tensor pipe is active 39%.  Measured
+// What bounds it: shared memory, where four operand stages fit.  The trispectrum
+// pass of 16 log bins at 256^3 takes 1,386 cycles per 64-point step, of which the
+// producers' and the accumulator warps' wavefronts fill 76% and the MMAs' operand
+// reads (128 + N rows of 32 bytes per 16 points) most of the rest; the tensor
+// pipe is active 42%.  Layouts of many rows have two or three stages: there the
+// wavefronts fill 49 to 54%, the tensor pipe is active 28 to 33% and the rest is
+// hand-off (the large levels of 192^3 x 48 and 384^3 x 29 linear bins).  Measured
 // against the tensor-memory kernel (CUDA events): 512^3, 16 log bins, triplets
 // and quadruplets 12.7 -> 8.5 ms; 64 log bins, triplets 7.7 -> 4.6 ms (its M =
 // 384 level, 18 bins and 32 pairs, 3.8 -> 1.8 ms, its M = 288 level, 57 bins
@@ -619,7 +622,7 @@ static void finish_gram(Plan &p, GramJob &job, const std::vector<GramRows> &grou
     job.usable = true;
 }
 
-// The rows' factors are 16-bit byte offsets into a field stage.
+// A field stage (the bins, a row of ones, a row of zeros) within 64 KB.
 static bool gram_bins(const Plan &p) { return p.nbins >= 1 && (p.nbins + 2) * kPts * 4 <= 65536; }
 
 static void build_gram_trip(Plan &p, GramJob &job) {

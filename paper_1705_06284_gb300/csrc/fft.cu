@@ -310,9 +310,8 @@ __global__ void __launch_bounds__(kThreads) inv_z_kernel(const typename V2<T>::t
     if (y0 >= nrows) return;
     T *ob = out + (long long)bl * out_bin_stride;
     if (g.empty) {
-        // shell fields: an empty bin's rows are never read by any item (its
-        // sum-of-squares partials stay at their zeroed value); count fields
-        // of the octant are zero-filled
+        // shell fields: levels hold no empty bin (nobody zeroes its rows or its
+        // sum-of-squares partials); count fields of the octant are zero-filled
         if (OCT) {
             const int H = N / 2 + 1;
             for (int i = threadIdx.x; i < nl * 2 * H; i += blockDim.x) {
